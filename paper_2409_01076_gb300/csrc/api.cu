@@ -434,7 +434,18 @@ int smrt_step(smrt_t *h, long long n)
     for (long long s = 0; s < n; ++s) {
         cudaError_t e;
         p.t = h->t;
-        if (h->layout == SMRT_LAYOUT_AB) {
+        // two-buffer float formats: three updates per pass over memory, the rest of n by twos (a single
+        // update moves as much memory as a pass of three)
+        const long long left = n - s;
+        const int k = (left >= 5 || left == 3) ? 3 : (left >= 2 ? 2 : 1);
+        if (h->layout == SMRT_LAYOUT_AB && T.sweep && k >= 2 && h->nx >= 8 && h->ny >= 8) {
+            e = T.sweep(h->collision, k, h->buf[h->cur], h->buf[1 - h->cur], p, h->stream);
+            if (e == cudaSuccess) {
+                h->cur = 1 - h->cur;
+                h->t += k - 1;
+                s += k - 1;
+            }
+        } else if (h->layout == SMRT_LAYOUT_AB) {
             e = T.step(h->collision, MODE_AB, h->buf[h->cur], h->buf[1 - h->cur], p, h->stream);
             if (e == cudaSuccess) h->cur = 1 - h->cur;
         } else {

@@ -302,9 +302,13 @@ struct WeightMul<float, true> {
 //   s = (+,-,+,-) over a = 1..4 (P = Pxx) and over a = 5..8 (P = Pxy), f*_0 = f^eq_0.
 // SRT (Eq. lb.srt): f*_a = f_a - (f_a - f^eq_a) / tau.
 // Two-tau (Eq. SmrtLBM-lb.1.5): f*_a = f_a - (f_a - f^eq_a)/tau_s + s_a (1/tau_s - 1/tau)/4 P.
-template <int KIND, bool EXACT = true, class C>
-__device__ __forceinline__ bool collide(const Params<C> &p, C g[9])
+//
+// The double form is written as plain expressions; the float form (collide_v below) spells out every
+// rounding, for one node or for two at a time, so that every kernel gets the same bits from it.
+template <int KIND, bool EXACT = true>
+__device__ __forceinline__ bool collide(const Params<double> &p, double g[9])
 {
+    using C = double;
     using M = WeightMul<C, EXACT>;
     const C drho = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
     const C rho = C(1) + drho;
@@ -364,6 +368,231 @@ __device__ __forceinline__ bool collide(const Params<C> &p, C g[9])
         g[8] -= txy;
     }
     return ok;
+}
+
+// ---- float arithmetic, one or two nodes at a time ----------------------------------
+// F2 holds the values of two nodes in a register pair; its operations are the packed add, sub, mul
+// and fma of this architecture: one instruction rounds both halves like the scalar one, so a node
+// gets the same bits either way at half the issue slots (the FMA rate is the same).
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float lo, float hi)
+{
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float f2_lo(F2 x)
+{
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x.v));
+    return lo;
+}
+__device__ __forceinline__ float f2_hi(F2 x)
+{
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x.v));
+    return hi;
+}
+__device__ __forceinline__ F2 vadd(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vsub(F2 a, F2 b)
+{
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vmul(F2 a, F2 b)
+{
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c)
+{
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+template <class V> __device__ __forceinline__ V vset(float c);
+template <> __device__ __forceinline__ float vset<float>(float c) { return c; }
+template <> __device__ __forceinline__ F2 vset<F2>(float c) { return f2(c, c); }
+
+// Four nodes, two by two: written so that the two halves' operations alternate.
+struct F4 {
+    F2 a, b;
+};
+__device__ __forceinline__ F4 vadd(F4 x, F4 y) { return {vadd(x.a, y.a), vadd(x.b, y.b)}; }
+__device__ __forceinline__ F4 vsub(F4 x, F4 y) { return {vsub(x.a, y.a), vsub(x.b, y.b)}; }
+__device__ __forceinline__ F4 vmul(F4 x, F4 y) { return {vmul(x.a, y.a), vmul(x.b, y.b)}; }
+__device__ __forceinline__ F4 vfma(F4 x, F4 y, F4 z) { return {vfma(x.a, y.a, z.a), vfma(x.b, y.b, z.b)}; }
+__device__ __forceinline__ F4 vsub(F2 x, F4 y) { return {vsub(x, y.a), vsub(x, y.b)}; }
+__device__ __forceinline__ F4 vmul(F2 x, F4 y) { return {vmul(x, y.a), vmul(x, y.b)}; }
+__device__ __forceinline__ F4 vfma(F2 x, F4 y, F4 z) { return {vfma(x, y.a, z.a), vfma(x, y.b, z.b)}; }
+
+// 1 / rho from -rho, correctly rounded wherever rho and 1 / rho are normal: the hardware's
+// approximation, good to one unit in the last place, and one Newton step with an exact residual,
+// which Markstein (1990) shows to round correctly (compared with the division for every float with
+// an exponent from 2^-126 to 2^125: equal).  The division's own sequence has a branch per node, for the
+// other operands, that keeps the nodes of a thread from overlapping.  Where rho is zero, infinite or
+// NaN the node has diverged and the result is NaN.
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float vrecip_neg(float nrho, float one)
+{
+    const float r = rcp_approx(-nrho);
+    return vfma(r, vfma(nrho, r, one), r);
+}
+__device__ __forceinline__ F2 vrecip_neg(F2 nrho, F2 one)
+{
+    const F2 r = f2(rcp_approx(-f2_lo(nrho)), rcp_approx(-f2_hi(nrho)));
+    return vfma(r, vfma(nrho, r, one), r);
+}
+
+__device__ __forceinline__ F4 vrecip_neg(F4 nrho, F2 one)
+{
+    const F4 r = {f2(rcp_approx(-f2_lo(nrho.a)), rcp_approx(-f2_hi(nrho.a))),
+                  f2(rcp_approx(-f2_lo(nrho.b)), rcp_approx(-f2_hi(nrho.b)))};
+    const F4 e = {vfma(nrho.a, r.a, one), vfma(nrho.b, r.b, one)};
+    return vfma(r, e, r);
+}
+
+// The constants of collide_v.  Two nodes at a time they are kernel arguments, so that the packed
+// instructions take them from there and need no register pair (nor the moves that fill one) for each.
+template <class V>
+struct CollideConsts {
+    V m1, p1, m15, c45, p3, m3;          // -1, 1, -3/2, 9/2, 3, -3
+    V hi[3], lo[3], mhi[3];              // the weights of the rest, axis and diagonal populations: w = hi + lo, and -hi
+    V r, s, t;                           // relaxation: -1/tau (SRT) or -1/tau_s (two-tau); +-(the P factor)
+};
+__host__ __device__ __forceinline__ void cc_set(float &v, float c) { v = c; }
+__host__ __device__ __forceinline__ void cc_set(F2 &v, float c)
+{
+    union { float f[2]; unsigned long long u; } w = {{c, c}};
+    v.v = w.u;
+}
+template <int KIND, class V>
+__host__ __device__ __forceinline__ CollideConsts<V> collide_consts(const Params<float> &p)
+{
+    CollideConsts<V> k;
+    cc_set(k.m1, -1.0f);
+    cc_set(k.p1, 1.0f);
+    cc_set(k.m15, -1.5f);
+    cc_set(k.c45, 4.5f);
+    cc_set(k.p3, 3.0f);
+    cc_set(k.m3, -3.0f);
+    for (int x = 0; x < 3; ++x) {
+        const double w = wgt<double>(x == 0 ? 0 : x == 1 ? 1 : 5);
+        const float hi = (float)w;
+        cc_set(k.hi[x], hi);
+        cc_set(k.lo[x], (float)(w - (double)hi));
+        cc_set(k.mhi[x], -hi);
+    }
+    const float f = KIND == SMRT_COLLISION_SMRT ? p.a4 : p.trt4;
+    cc_set(k.r, KIND == SMRT_COLLISION_SRT ? -p.omega : -p.omega_s);
+    cc_set(k.s, f);
+    cc_set(k.t, -f);
+    return k;
+}
+
+template <bool SPLIT>
+__device__ __forceinline__ float vfma_last(int, float a, float b, float c) { return vfma(a, b, c); }
+template <bool SPLIT>
+__device__ __forceinline__ F2 vfma_last(int dir, F2 a, F2 b, F2 c)
+{
+    if (SPLIT && ex(dir) != 0)
+        return f2(__fmaf_rn(f2_lo(a), f2_lo(b), f2_lo(c)), __fmaf_rn(f2_hi(a), f2_hi(b), f2_hi(c)));
+    return vfma(a, b, c);
+}
+
+template <bool SPLIT>
+__device__ __forceinline__ F4 vfma_last(int dir, F2 a, F4 b, F4 c)
+{
+    return {vfma_last<SPLIT>(dir, a, b.a, c.a), vfma_last<SPLIT>(dir, a, b.b, c.b)};
+}
+template <class V> struct ConstOf { using type = V; };
+template <> struct ConstOf<F4> { using type = F2; };
+
+// The same collision on V = float or F2, every operation rounded as written.  Returns -rho.
+// EXACT: the weight products are those of WeightMul<float, true>; otherwise they are plain, and fused
+// with the operation that follows.  SPLIT: the last operation of the populations that move along x works
+// on each half by itself: its caller regroups the halves for the shift, and a scalar result lands in
+// either half of a register pair without a move.
+template <int KIND, bool EXACT, bool SPLIT, class V>
+__device__ __forceinline__ V collide_v(const CollideConsts<typename ConstOf<V>::type> &k, V g[9])
+{
+    const V drho = vadd(vadd(vadd(vadd(g[0], g[1]), vadd(g[2], g[3])),
+                             vadd(vadd(g[4], g[5]), vadd(g[6], g[7]))), g[8]);
+    const V nrho = vsub(k.m1, drho);
+    const V jx = vadd(vadd(vsub(g[1], g[3]), vsub(g[5], g[6])), vsub(g[8], g[7]));
+    const V jy = vsub(vadd(vsub(g[2], g[4]), vadd(g[5], g[6])), vadd(g[7], g[8]));
+    const V inv = vrecip_neg(nrho, k.p1);
+    const V ux = vmul(jx, inv), uy = vmul(jy, inv);
+    const V base = vfma(k.m15, vfma(jx, ux, vmul(jy, uy)), drho);
+    const V jp = vadd(jx, jy), jm = vsub(jx, jy);
+    const V up = vadd(ux, uy), um = vsub(ux, uy);
+    const V axx = vfma(vmul(k.c45, jx), ux, base), ayy = vfma(vmul(k.c45, jy), uy, base);
+    const V app = vfma(vmul(k.c45, jp), up, base), amm = vfma(vmul(k.c45, jm), um, base);
+    // q_a = w_a x_a
+    const V x[9] = {base, vfma(k.p3, jx, axx), vfma(k.p3, jy, ayy), vfma(k.m3, jx, axx), vfma(k.m3, jy, ayy),
+                    vfma(k.p3, jp, app), vfma(k.m3, jm, amm), vfma(k.m3, jp, app), vfma(k.p3, jm, amm)};
+    V q[9], n[9];
+    #pragma unroll
+    for (int a = 0; a < 9; ++a) {
+        const int w = a == 0 ? 0 : a < 5 ? 1 : 2;
+        if (EXACT) {
+            q[a] = vfma(k.hi[w], x[a], vmul(k.lo[w], x[a]));
+            n[a] = vsub(g[a], q[a]);
+        } else {
+            n[a] = vfma(k.mhi[w], x[a], g[a]);
+        }
+    }
+    if (KIND == SMRT_COLLISION_SRT) {
+        #pragma unroll
+        for (int a = 0; a < 9; ++a) g[a] = vfma_last<SPLIT>(a, k.r, n[a], g[a]);
+        return nrho;
+    }
+    const V pxx = vsub(vadd(n[1], n[3]), vadd(n[2], n[4]));
+    const V pxy = vsub(vadd(n[5], n[7]), vadd(n[6], n[8]));
+    if (KIND == SMRT_COLLISION_SMRT) {
+        if (EXACT) {
+            g[0] = q[0];
+            #pragma unroll
+            for (int a = 1; a < 9; ++a) g[a] = vfma_last<SPLIT>(a, (a & 1) ? k.s : k.t, a < 5 ? pxx : pxy, q[a]);
+        } else {
+            const V txx = vmul(k.s, pxx), txy = vmul(k.s, pxy), sxx = vmul(k.t, pxx), sxy = vmul(k.t, pxy);
+            g[0] = vmul(k.hi[0], x[0]);
+            #pragma unroll
+            for (int a = 1; a < 9; ++a)
+                g[a] = vfma_last<SPLIT>(a, k.hi[a < 5 ? 1 : 2], x[a],
+                                        a < 5 ? ((a & 1) ? txx : sxx) : ((a & 1) ? txy : sxy));
+        }
+    } else {
+        g[0] = vfma(k.r, n[0], g[0]);
+        #pragma unroll
+        for (int a = 1; a < 9; ++a) g[a] = vfma_last<SPLIT>(a, (a & 1) ? k.s : k.t, a < 5 ? pxx : pxy, vfma(k.r, n[a], g[a]));
+    }
+    return nrho;
+}
+
+template <int KIND, bool EXACT = true>
+__device__ __forceinline__ bool collide(const Params<float> &p, float g[9])
+{
+    const float nrho = collide_v<KIND, EXACT, false, float>(collide_consts<KIND, float>(p), g);
+    return nrho < 0.0f && nrho > -INFINITY;
 }
 
 } // namespace smrt

@@ -51,6 +51,8 @@ constexpr int kResidualMaxBlocks = 1216; // 8 x 152 SMs
 struct KernelTable {
     cudaError_t (*step)(int kind, int mode, const void *src, void *dst, const HostParams &p,
                         cudaStream_t s);
+    // 2 or 3 updates in one launch, two-buffer layout, nx >= 8 and ny >= 8 (null: not for this precision)
+    cudaError_t (*sweep)(int kind, int updates, const void *src, void *dst, const HostParams &p, cudaStream_t s);
     cudaError_t (*get_f)(int mode, const void *state, double *f, int row0, int rows,
                          const HostParams &p, cudaStream_t s);
     cudaError_t (*set_f)(int mode, void *state, const double *f, int row0, int rows,

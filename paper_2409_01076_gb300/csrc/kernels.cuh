@@ -16,6 +16,7 @@
 #pragma once
 
 #include "d2q9.cuh"
+#include "sweep.cuh"
 
 namespace smrt {
 
@@ -884,6 +885,71 @@ cudaError_t launch_step(int kind, int mode, const void *src, void *dst, const Ho
     }
 }
 
+// T updates in one pass (sweep.cuh).  Rows per segment: the rows that two segments share are computed
+// twice, so long segments do less work, but a lattice that gives each of the 608 SM sub-partitions few
+// warps is bound by the latency of one warp's walk.  Measured (f32, T = 3, 64^2 to 8192^2): a row of one
+// update takes a warp max(0.685, 0.35 + 0.30 w) us with w warps per sub-partition, w also standing for
+// the waves beyond the 4 resident; the minimum of (rows + T - 1) x that is within 4 % of the best of a
+// sweep over rows at every size.  (64^2: 1 row, 6.2 us per single update -> 4.1; 1024^2: 6, 12.3 -> 10.9;
+// 4096^2: 20, 178 -> 88; 8192^2: 64, 694 -> 290.)
+inline int sweep_rows(int strips, int ny, int T)
+{
+    int best = 1;
+    double least = 1e300;
+    for (int rows = 1; rows <= 64 && rows <= ny; ++rows) {
+        const double w = (double)strips * ((ny + rows - 1) / rows) / 608.0;
+        const double one = 0.35 + 0.30 * w;
+        const double cost = (rows + T - 1) * (one > 0.685 ? one : 0.685);
+        if (cost < least) {
+            least = cost;
+            best = rows;
+        }
+    }
+    return best;
+}
+
+template <int PREC, int KIND, int T>
+cudaError_t launch_sweep_kt(const void *src, void *dst, const HostParams &hp, cudaStream_t s)
+{
+    using P = Prec<PREC>;
+    using R = typename P::R;
+    const Params<typename P::C> p = make_params<typename P::C>(hp);
+    const CollideConsts<F2> cc = collide_consts<KIND, F2>(p);
+    SweepSalts<T> salt;
+    for (int m = 0; m < T; ++m) salt.s[m] = sr_salt(hp.t + m);
+    const int strips = (hp.nx + kSwOwn - 1) / kSwOwn, rows = sweep_rows(strips, hp.ny, T);
+    const unsigned nb = (unsigned)((long long)strips * ((hp.ny + rows - 1) / rows));
+    if constexpr (PREC == SMRT_PREC_F16 || PREC == SMRT_PREC_BF16) {
+        if (hp.rounding == SMRT_ROUND_STOCHASTIC) {
+            sweep_kernel<PREC, KIND, true, T><<<nb, 32, 0, s>>>((const R *)src, (R *)dst, p, cc, salt, strips, rows);
+            return cudaGetLastError();
+        }
+    }
+    sweep_kernel<PREC, KIND, false, T><<<nb, 32, 0, s>>>((const R *)src, (R *)dst, p, cc, salt, strips, rows);
+    return cudaGetLastError();
+}
+
+template <int PREC, int KIND>
+cudaError_t launch_sweep_k(int updates, const void *src, void *dst, const HostParams &hp, cudaStream_t s)
+{
+    switch (updates) {
+    case 2: return launch_sweep_kt<PREC, KIND, 2>(src, dst, hp, s);
+    case 3: return launch_sweep_kt<PREC, KIND, 3>(src, dst, hp, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+template <int PREC>
+cudaError_t launch_sweep(int kind, int updates, const void *src, void *dst, const HostParams &hp, cudaStream_t s)
+{
+    switch (kind) {
+    case SMRT_COLLISION_SMRT: return launch_sweep_k<PREC, SMRT_COLLISION_SMRT>(updates, src, dst, hp, s);
+    case SMRT_COLLISION_SRT: return launch_sweep_k<PREC, SMRT_COLLISION_SRT>(updates, src, dst, hp, s);
+    case SMRT_COLLISION_TWO_TAU: return launch_sweep_k<PREC, SMRT_COLLISION_TWO_TAU>(updates, src, dst, hp, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 inline unsigned node_blocks(int rows, int nx, int threads)
 {
     long long n = (long long)rows * nx;
@@ -991,6 +1057,8 @@ KernelTable make_table()
 {
     KernelTable t;
     t.step = &launch_step<PREC>;
+    if constexpr (PREC != SMRT_PREC_F64) t.sweep = &launch_sweep<PREC>;
+    else t.sweep = nullptr;
     t.get_f = &launch_get_f<PREC>;
     t.set_f = &launch_set_f<PREC>;
     t.init_macros = &launch_init_macros<PREC>;
