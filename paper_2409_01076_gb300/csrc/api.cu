@@ -17,6 +17,7 @@ namespace {
 
 using smrt::HostParams;
 using smrt::KernelTable;
+using smrt::TilePlan;
 
 thread_local std::string g_create_error = "no error";
 
@@ -65,6 +66,7 @@ struct smrt_t {
     size_t stage_bytes = 0;
     size_t dev_bytes = 0;
     long long t = 0;
+    TilePlan tile = {};        // how smrt_step takes several updates per launch of a small lattice (T == 0: not)
     std::string err = "no error";
 };
 
@@ -162,6 +164,70 @@ HostParams host_params(const smrt_t *h)
     return p;
 }
 
+TilePlan tile_shape(int nx, int ny, int prec, int W, int H, int updates)
+{
+    TilePlan t;
+    t.W = W;
+    t.H = H;
+    t.T = updates;
+    t.tiles_x = (nx + W - 1) / W;
+    t.tiles_y = (ny + H - 1) / H;
+    const int area = (W + 2 * (updates - 1)) * (H + 2 * (updates - 1));
+    t.threads = area >= 512 ? 512 : (area + 31) / 32 * 32;
+    t.shared = (size_t)18 * area * elem_bytes(prec);
+    return t;
+}
+
+// Whether and how the two-buffer layout takes several updates per launch in tiles (T == 0: it does not).
+// A launch costs 6.2-6.5 us of latency whatever it does.  Beyond that an update of `warps` warps per block
+// and `blocks` / 152 blocks per SM was measured to take (64^2 to 1024^2, 40 plans each)
+//   double: 0.52 us x the warps per SM (the double pipe), at least the 1.75 us of one warp's chain,
+//   float:  0.45 us + 0.06 us x the warps per SM.
+// The alternatives: one update per launch in double, 3.2 + 0.52 us per warp of the SM; sweeps of three in
+// float (sweep_rows' model).  Measured, us per update, before -> after: 64^2 f64 10.3 -> 3.6 (8 x 4, T = 4),
+// 128^2 f64 8.2 -> 5.2 (16 x 8, T = 4), 64^2 f32 6.2 -> 1.6 (8 x 4, T = 8), 256^2 f32 6.2 -> 2.8 (16 x 16,
+// T = 6).  256^2 f64 (12.3 against 10.3 one by one) and 512^2 f32 (7.2 against 6.2 by sweeps) stay out.
+TilePlan tile_plan(int nx, int ny, int prec)
+{
+    TilePlan best;
+    best.T = 0;
+    if ((long long)nx * ny > 600LL * 600) return best;
+    const bool f64 = prec == SMRT_PREC_F64;
+    double least;
+    if (f64) {
+        least = 3.2 + 0.52 * ((double)nx * ny / 32.0 / 152.0);
+        if (least < 6.2) least = 6.2;
+    } else {
+        const int strips = nx <= 128 ? 1 : (nx + 111) / 120;
+        least = 1e300;
+        for (int rows = 1; rows <= 64 && rows <= ny; ++rows) {
+            const double one = 0.35 + 0.30 * ((double)strips * ((ny + rows - 1) / rows) / 608.0);
+            const double us = (6.0 + 3.0 * (rows + 2) * (one > 0.685 ? one : 0.685)) / 3.0;
+            if (us < least) least = us;
+        }
+    }
+    least *= 0.97;
+    const int side[] = {4, 8, 16, 24, 32}, updates[] = {2, 3, 4, 6, 8};
+    for (int T : updates)
+        for (int W : side)
+            for (int H : side) {
+                const TilePlan t = tile_shape(nx, ny, prec, W, H, T);
+                if (H > W || W + 2 * (T - 1) >= 64 || t.shared > 48 * 1024) continue;
+                const double per_sm = (double)t.tiles_x * t.tiles_y / 152.0;
+                double us = 6.4;
+                for (int ring = T - 1; ring >= 0; --ring) {
+                    const int warps = ((W + 2 * ring) * (H + 2 * ring) + 31) / 32;
+                    const double w = warps * (per_sm > 1.0 ? per_sm : 1.0);
+                    us += f64 ? (0.52 * w > 1.75 ? 0.52 * w : 1.75) : 0.45 + 0.06 * w;
+                }
+                if (us / T < least) {
+                    least = us / T;
+                    best = t;
+                }
+            }
+    return best;
+}
+
 int current_mode(const smrt_t *h)
 {
     if (h->layout == SMRT_LAYOUT_AB) return MODE_AB;
@@ -230,6 +296,7 @@ int materialize(smrt_t *h)
         release(h);
         return cuda_fail(h, e, "cudaMallocHost");
     }
+    h->tile = tile_plan(h->nx, h->ny, h->prec);
     h->ready = true;
     h->t = 0;
     h->cur = 0;
@@ -431,15 +498,24 @@ int smrt_step(smrt_t *h, long long n)
     CUDA_TRY(h, g.err);
     const KernelTable &T = table_for(h->prec);
     HostParams p = host_params(h);
+    const bool passes = h->layout == SMRT_LAYOUT_AB && n >= 2 && h->nx >= 8 && h->ny >= 8;
+    const TilePlan &tile = h->tile;
     for (long long s = 0; s < n; ++s) {
         cudaError_t e;
         p.t = h->t;
-        // two-buffer float formats: three updates per pass over memory, the rest of n by twos (a single
-        // update moves as much memory as a pass of three)
         const long long left = n - s;
-        const int k = (left >= 5 || left == 3) ? 3 : (left >= 2 ? 2 : 1);
-        if (h->layout == SMRT_LAYOUT_AB && T.sweep && k >= 2 && h->nx >= 8 && h->ny >= 8) {
-            e = T.sweep(h->collision, k, h->buf[h->cur], h->buf[1 - h->cur], p, h->stream);
+        if (passes && left >= 2 && (tile.T || T.sweep)) {
+            int k;
+            if (tile.T) {
+                TilePlan t = tile;
+                if (left < t.T) t = tile_shape(h->nx, h->ny, h->prec, t.W, t.H, (int)left);
+                k = t.T;
+                e = T.tile(h->collision, t, h->buf[h->cur], h->buf[1 - h->cur], p, h->stream);
+            } else {
+                // by threes, the rest by twos: a single update moves as much memory as a pass of three
+                k = (left >= 5 || left == 3) ? 3 : 2;
+                e = T.sweep(h->collision, k, h->buf[h->cur], h->buf[1 - h->cur], p, h->stream);
+            }
             if (e == cudaSuccess) {
                 h->cur = 1 - h->cur;
                 h->t += k - 1;

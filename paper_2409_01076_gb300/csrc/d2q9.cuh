@@ -140,6 +140,8 @@ struct Params {
     C omega_s;          // 1 / tau_s (two-relaxation-time form)
     C a4;               // (1 - 1/tau) / 4, SmrtLBM
     C trt4;             // (1/tau_s - 1/tau) / 4, two-relaxation-time form
+    C keep, keep_s;     // 1 - 1/tau, 1 - 1/tau_s       (the double collision)
+    C deq, deq_s;       // 1/4 - a4 = 1/(4 tau), 1/4 - tau_s trt4 = tau_s/(4 tau)   (the double collision)
     C corr[4][9];       // moving-wall term 6 w_a (e_a . u_w(side)) added to a wall-pulled offset
     int *flag;          // divergence flag (bit 0)
     uint32_t salt;      // stochastic rounding: the salt of this launch's time step
@@ -159,6 +161,10 @@ inline Params<C> make_params(const HostParams &h)
     p.omega_s = C(1.0 / h.tau_s);
     p.a4 = C((1.0 - 1.0 / h.tau) / 4.0);
     p.trt4 = C((1.0 / h.tau_s - 1.0 / h.tau) / 4.0);
+    p.keep = C(1.0 - 1.0 / h.tau);
+    p.keep_s = C(1.0 - 1.0 / h.tau_s);
+    p.deq = C(0.25 / h.tau);
+    p.deq_s = C(0.25 * h.tau_s / h.tau);
     for (int s = 0; s < 4; ++s) {
         unsigned kind = (h.bc >> (2 * s)) & 3u;
         double wx = 0.0, wy = 0.0;
@@ -303,12 +309,277 @@ struct WeightMul<float, true> {
 // SRT (Eq. lb.srt): f*_a = f_a - (f_a - f^eq_a) / tau.
 // Two-tau (Eq. SmrtLBM-lb.1.5): f*_a = f_a - (f_a - f^eq_a)/tau_s + s_a (1/tau_s - 1/tau)/4 P.
 //
-// The double form is written as plain expressions; the float form (collide_v below) spells out every
-// rounding, for one node or for two at a time, so that every kernel gets the same bits from it.
+// Double: this GPU starts a warp's double operation every 64 clocks per SM sub-partition, so their number is
+// the kernel's time.  With the even and odd parts of each opposite pair, K = j.u, D = jx ux - jy uy and
+// jx uy, the equilibrium is
+//   f^eq_0 - w_0 = 4/9 drho - 2/3 K,   axes: drho/9 + K/12 +- D/4 +- j/3,   diagonals: drho/36 + K/12 +- jx uy/4
+//   +- (jx +- jy)/12,
+// and its P^eq are D and jx uy themselves, so the collision needs 52 operations (SmrtLBM) where the
+// populations one by one took 75: 4096^2 2.31 -> 1.62 ms per update, 10.4 G updates/s.  1/rho is the hardware's approximation
+// (20 bits) and one step of Halley's iteration, within one unit in the last place of the division; the
+// check of rho works on its upper word.
+__device__ __forceinline__ double recip_d(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
 template <int KIND, bool EXACT = true>
 __device__ __forceinline__ bool collide(const Params<double> &p, double g[9])
 {
-    using C = double;
+    const double s13 = g[1] + g[3], s24 = g[2] + g[4], s57 = g[5] + g[7], s68 = g[6] + g[8];
+    const double d13 = g[1] - g[3], d24 = g[2] - g[4], d57 = g[5] - g[7], d68 = g[6] - g[8];
+    double drho = g[0] + ((s13 + s24) + (s57 + s68));
+    const double rho = 1.0 + drho;
+    double jx = d13 + (d57 - d68), jy = d24 + (d57 + d68);
+    const double inv = recip_d(rho);
+    const double ux = jx * inv, uy = jy * inv;
+    const int hi = __double2hiint(rho);
+    const bool ok = (unsigned)hi < 0x7ff00000u && (hi | __double2loint(rho)) != 0;
+    if (KIND != SMRT_COLLISION_SMRT) {          // the equilibrium's share of f*
+        const double o = KIND == SMRT_COLLISION_SRT ? p.omega : p.omega_s;
+        drho *= o;
+        jx *= o;
+        jy *= o;
+    }
+    const double xx = jx * ux, yy = jy * uy, xy = jx * uy;
+    const double K = xx + yy, D = xx - yy, k12 = K * (1.0 / 12.0);
+    double n, m;                                 // what P adds to the axes and the diagonals
+    if (KIND == SMRT_COLLISION_SMRT) {
+        n = fma(p.a4, s13 - s24, p.deq * D);
+        m = fma(p.a4, s57 - s68, p.deq * xy);
+    } else if (KIND == SMRT_COLLISION_SRT) {
+        n = 0.25 * D;
+        m = 0.25 * xy;
+    } else {
+        n = fma(p.trt4, s13 - s24, p.deq_s * D);
+        m = fma(p.trt4, s57 - s68, p.deq_s * xy);
+    }
+    const double a = fma(drho, 1.0 / 9.0, k12), b = fma(drho, 1.0 / 36.0, k12);
+    const double ax = a + n, ay = a - n, bp = b + m, bm = b - m;
+    const double jp = jx + jy, jm = jx - jy;
+    const double q0 = fma(drho, 4.0 / 9.0, K * (-2.0 / 3.0));
+    const double q1 = fma(jx, 1.0 / 3.0, ax), q3 = fma(jx, -1.0 / 3.0, ax);
+    const double q2 = fma(jy, 1.0 / 3.0, ay), q4 = fma(jy, -1.0 / 3.0, ay);
+    const double q5 = fma(jp, 1.0 / 12.0, bp), q7 = fma(jp, -1.0 / 12.0, bp);
+    const double q8 = fma(jm, 1.0 / 12.0, bm), q6 = fma(jm, -1.0 / 12.0, bm);
+    const double q[9] = {q0, q1, q2, q3, q4, q5, q6, q7, q8};
+    #pragma unroll
+    for (int k = 0; k < 9; ++k)
+        g[k] = KIND == SMRT_COLLISION_SMRT ? q[k] : fma(KIND == SMRT_COLLISION_SRT ? p.keep : p.keep_s, g[k], q[k]);
+    return ok;
+}
+
+// ---- float arithmetic, one or two nodes at a time ----------------------------------
+// F2 holds the values of two nodes in a register pair; its operations are the packed add, sub, mul
+// and fma of this architecture: one instruction rounds both halves like the scalar one, so a node
+// gets the same bits either way at half the issue slots (the FMA rate is the same).
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float lo, float hi)
+{
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float f2_lo(F2 x)
+{
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x.v));
+    return lo;
+}
+__device__ __forceinline__ float f2_hi(F2 x)
+{
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x.v));
+    return hi;
+}
+__device__ __forceinline__ F2 vadd(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vsub(F2 a, F2 b)
+{
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vmul(F2 a, F2 b)
+{
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c)
+{
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+template <class V> __device__ __forceinline__ V vset(float c);
+template <> __device__ __forceinline__ F2 vset<F2>(float c) { return f2(c, c); }
+
+// Four nodes, two by two: written so that the two halves' operations alternate.
+struct F4 {
+    F2 a, b;
+};
+__device__ __forceinline__ F4 vadd(F4 x, F4 y) { return {vadd(x.a, y.a), vadd(x.b, y.b)}; }
+__device__ __forceinline__ F4 vsub(F4 x, F4 y) { return {vsub(x.a, y.a), vsub(x.b, y.b)}; }
+__device__ __forceinline__ F4 vmul(F4 x, F4 y) { return {vmul(x.a, y.a), vmul(x.b, y.b)}; }
+__device__ __forceinline__ F4 vfma(F4 x, F4 y, F4 z) { return {vfma(x.a, y.a, z.a), vfma(x.b, y.b, z.b)}; }
+__device__ __forceinline__ F4 vsub(F2 x, F4 y) { return {vsub(x, y.a), vsub(x, y.b)}; }
+__device__ __forceinline__ F4 vmul(F2 x, F4 y) { return {vmul(x, y.a), vmul(x, y.b)}; }
+__device__ __forceinline__ F4 vfma(F2 x, F4 y, F4 z) { return {vfma(x, y.a, z.a), vfma(x, y.b, z.b)}; }
+
+// 1 / rho from -rho, correctly rounded wherever rho and 1 / rho are normal: the hardware's
+// approximation, good to one unit in the last place, and one Newton step with an exact residual,
+// which Markstein (1990) shows to round correctly (compared with the division for every float with
+// an exponent from 2^-126 to 2^125: equal).  The division's own sequence has a branch per node, for the
+// other operands, that keeps the nodes of a thread from overlapping.  Where rho is zero, infinite or
+// NaN the node has diverged and the result is NaN.
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ F2 vrecip_neg(F2 nrho, F2 one)
+{
+    const F2 r = f2(rcp_approx(-f2_lo(nrho)), rcp_approx(-f2_hi(nrho)));
+    return vfma(r, vfma(nrho, r, one), r);
+}
+
+__device__ __forceinline__ F4 vrecip_neg(F4 nrho, F2 one)
+{
+    const F4 r = {f2(rcp_approx(-f2_lo(nrho.a)), rcp_approx(-f2_hi(nrho.a))),
+                  f2(rcp_approx(-f2_lo(nrho.b)), rcp_approx(-f2_hi(nrho.b)))};
+    const F4 e = {vfma(nrho.a, r.a, one), vfma(nrho.b, r.b, one)};
+    return vfma(r, e, r);
+}
+
+// The constants of collide_v are kernel arguments, so that the packed
+// instructions take them from there and need no register pair (nor the moves that fill one) for each.
+struct CollideConsts {
+    F2 m1, p1, m15, c45, p3, m3;          // -1, 1, -3/2, 9/2, 3, -3
+    F2 hi[3], lo[3], mhi[3];              // the weights of the rest, axis and diagonal populations: w = hi + lo, and -hi
+    F2 r, s, t;                          // relaxation: -1/tau (SRT) or -1/tau_s (two-tau); +-(the P factor)
+};
+inline void cc_set(F2 &v, float c)
+{
+    union { float f[2]; unsigned long long u; } w = {{c, c}};
+    v.v = w.u;
+}
+template <int KIND>
+inline CollideConsts collide_consts(const Params<float> &p)
+{
+    CollideConsts k;
+    cc_set(k.m1, -1.0f);
+    cc_set(k.p1, 1.0f);
+    cc_set(k.m15, -1.5f);
+    cc_set(k.c45, 4.5f);
+    cc_set(k.p3, 3.0f);
+    cc_set(k.m3, -3.0f);
+    for (int x = 0; x < 3; ++x) {
+        const double w = wgt<double>(x == 0 ? 0 : x == 1 ? 1 : 5);
+        const float hi = (float)w;
+        cc_set(k.hi[x], hi);
+        cc_set(k.lo[x], (float)(w - (double)hi));
+        cc_set(k.mhi[x], -hi);
+    }
+    const float f = KIND == SMRT_COLLISION_SMRT ? p.a4 : p.trt4;
+    cc_set(k.r, KIND == SMRT_COLLISION_SRT ? -p.omega : -p.omega_s);
+    cc_set(k.s, f);
+    cc_set(k.t, -f);
+    return k;
+}
+
+template <bool SPLIT>
+__device__ __forceinline__ F2 vfma_last(int dir, F2 a, F2 b, F2 c)
+{
+    if (SPLIT && ex(dir) != 0)
+        return f2(__fmaf_rn(f2_lo(a), f2_lo(b), f2_lo(c)), __fmaf_rn(f2_hi(a), f2_hi(b), f2_hi(c)));
+    return vfma(a, b, c);
+}
+
+template <bool SPLIT>
+__device__ __forceinline__ F4 vfma_last(int dir, F2 a, F4 b, F4 c)
+{
+    return {vfma_last<SPLIT>(dir, a, b.a, c.a), vfma_last<SPLIT>(dir, a, b.b, c.b)};
+}
+// The collision of float populations on F4, every operation rounded as written.  Returns -rho.
+// EXACT: the weight products are those of WeightMul<float, true>; otherwise they are plain, and fused
+// with the operation that follows.  SPLIT: the last operation of the populations that move along x works
+// on each half by itself: its caller regroups the halves for the shift, and a scalar result lands in
+// either half of a register pair without a move.
+template <int KIND, bool EXACT, bool SPLIT>
+__device__ __forceinline__ F4 collide_v(const CollideConsts &k, F4 g[9])
+{
+    using V = F4;
+    const V drho = vadd(vadd(vadd(vadd(g[0], g[1]), vadd(g[2], g[3])),
+                             vadd(vadd(g[4], g[5]), vadd(g[6], g[7]))), g[8]);
+    const V nrho = vsub(k.m1, drho);
+    const V jx = vadd(vadd(vsub(g[1], g[3]), vsub(g[5], g[6])), vsub(g[8], g[7]));
+    const V jy = vsub(vadd(vsub(g[2], g[4]), vadd(g[5], g[6])), vadd(g[7], g[8]));
+    const V inv = vrecip_neg(nrho, k.p1);
+    const V ux = vmul(jx, inv), uy = vmul(jy, inv);
+    const V base = vfma(k.m15, vfma(jx, ux, vmul(jy, uy)), drho);
+    const V jp = vadd(jx, jy), jm = vsub(jx, jy);
+    const V up = vadd(ux, uy), um = vsub(ux, uy);
+    const V axx = vfma(vmul(k.c45, jx), ux, base), ayy = vfma(vmul(k.c45, jy), uy, base);
+    const V app = vfma(vmul(k.c45, jp), up, base), amm = vfma(vmul(k.c45, jm), um, base);
+    // q_a = w_a x_a
+    const V x[9] = {base, vfma(k.p3, jx, axx), vfma(k.p3, jy, ayy), vfma(k.m3, jx, axx), vfma(k.m3, jy, ayy),
+                    vfma(k.p3, jp, app), vfma(k.m3, jm, amm), vfma(k.m3, jp, app), vfma(k.p3, jm, amm)};
+    V q[9], n[9];
+    #pragma unroll
+    for (int a = 0; a < 9; ++a) {
+        const int w = a == 0 ? 0 : a < 5 ? 1 : 2;
+        if (EXACT) {
+            q[a] = vfma(k.hi[w], x[a], vmul(k.lo[w], x[a]));
+            n[a] = vsub(g[a], q[a]);
+        } else {
+            n[a] = vfma(k.mhi[w], x[a], g[a]);
+        }
+    }
+    if (KIND == SMRT_COLLISION_SRT) {
+        #pragma unroll
+        for (int a = 0; a < 9; ++a) g[a] = vfma_last<SPLIT>(a, k.r, n[a], g[a]);
+        return nrho;
+    }
+    const V pxx = vsub(vadd(n[1], n[3]), vadd(n[2], n[4]));
+    const V pxy = vsub(vadd(n[5], n[7]), vadd(n[6], n[8]));
+    if (KIND == SMRT_COLLISION_SMRT) {
+        if (EXACT) {
+            g[0] = q[0];
+            #pragma unroll
+            for (int a = 1; a < 9; ++a) g[a] = vfma_last<SPLIT>(a, (a & 1) ? k.s : k.t, a < 5 ? pxx : pxy, q[a]);
+        } else {
+            const V txx = vmul(k.s, pxx), txy = vmul(k.s, pxy), sxx = vmul(k.t, pxx), sxy = vmul(k.t, pxy);
+            g[0] = vmul(k.hi[0], x[0]);
+            #pragma unroll
+            for (int a = 1; a < 9; ++a)
+                g[a] = vfma_last<SPLIT>(a, k.hi[a < 5 ? 1 : 2], x[a],
+                                        a < 5 ? ((a & 1) ? txx : sxx) : ((a & 1) ? txy : sxy));
+        }
+    } else {
+        g[0] = vfma(k.r, n[0], g[0]);
+        #pragma unroll
+        for (int a = 1; a < 9; ++a) g[a] = vfma_last<SPLIT>(a, (a & 1) ? k.s : k.t, a < 5 ? pxx : pxy, vfma(k.r, n[a], g[a]));
+    }
+    return nrho;
+}
+
+// One node by plain expressions, which the compiler contracts to the operations of collide_v (compared bit for
+// bit): for the kernels bound by memory, where this form measured 2-4 % faster in 16-bit storage.
+template <int KIND, bool EXACT = true>
+__device__ __forceinline__ bool collide(const Params<float> &p, float g[9])
+{
+    using C = float;
     using M = WeightMul<C, EXACT>;
     const C drho = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
     const C rho = C(1) + drho;
@@ -368,231 +639,6 @@ __device__ __forceinline__ bool collide(const Params<double> &p, double g[9])
         g[8] -= txy;
     }
     return ok;
-}
-
-// ---- float arithmetic, one or two nodes at a time ----------------------------------
-// F2 holds the values of two nodes in a register pair; its operations are the packed add, sub, mul
-// and fma of this architecture: one instruction rounds both halves like the scalar one, so a node
-// gets the same bits either way at half the issue slots (the FMA rate is the same).
-struct F2 {
-    unsigned long long v;
-};
-__device__ __forceinline__ F2 f2(float lo, float hi)
-{
-    F2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float f2_lo(F2 x)
-{
-    float lo, hi;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x.v));
-    return lo;
-}
-__device__ __forceinline__ float f2_hi(F2 x)
-{
-    float lo, hi;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x.v));
-    return hi;
-}
-__device__ __forceinline__ F2 vadd(F2 a, F2 b)
-{
-    F2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ F2 vsub(F2 a, F2 b)
-{
-    F2 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ F2 vmul(F2 a, F2 b)
-{
-    F2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c)
-{
-    F2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-    return r;
-}
-__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-template <class V> __device__ __forceinline__ V vset(float c);
-template <> __device__ __forceinline__ float vset<float>(float c) { return c; }
-template <> __device__ __forceinline__ F2 vset<F2>(float c) { return f2(c, c); }
-
-// Four nodes, two by two: written so that the two halves' operations alternate.
-struct F4 {
-    F2 a, b;
-};
-__device__ __forceinline__ F4 vadd(F4 x, F4 y) { return {vadd(x.a, y.a), vadd(x.b, y.b)}; }
-__device__ __forceinline__ F4 vsub(F4 x, F4 y) { return {vsub(x.a, y.a), vsub(x.b, y.b)}; }
-__device__ __forceinline__ F4 vmul(F4 x, F4 y) { return {vmul(x.a, y.a), vmul(x.b, y.b)}; }
-__device__ __forceinline__ F4 vfma(F4 x, F4 y, F4 z) { return {vfma(x.a, y.a, z.a), vfma(x.b, y.b, z.b)}; }
-__device__ __forceinline__ F4 vsub(F2 x, F4 y) { return {vsub(x, y.a), vsub(x, y.b)}; }
-__device__ __forceinline__ F4 vmul(F2 x, F4 y) { return {vmul(x, y.a), vmul(x, y.b)}; }
-__device__ __forceinline__ F4 vfma(F2 x, F4 y, F4 z) { return {vfma(x, y.a, z.a), vfma(x, y.b, z.b)}; }
-
-// 1 / rho from -rho, correctly rounded wherever rho and 1 / rho are normal: the hardware's
-// approximation, good to one unit in the last place, and one Newton step with an exact residual,
-// which Markstein (1990) shows to round correctly (compared with the division for every float with
-// an exponent from 2^-126 to 2^125: equal).  The division's own sequence has a branch per node, for the
-// other operands, that keeps the nodes of a thread from overlapping.  Where rho is zero, infinite or
-// NaN the node has diverged and the result is NaN.
-__device__ __forceinline__ float rcp_approx(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float vrecip_neg(float nrho, float one)
-{
-    const float r = rcp_approx(-nrho);
-    return vfma(r, vfma(nrho, r, one), r);
-}
-__device__ __forceinline__ F2 vrecip_neg(F2 nrho, F2 one)
-{
-    const F2 r = f2(rcp_approx(-f2_lo(nrho)), rcp_approx(-f2_hi(nrho)));
-    return vfma(r, vfma(nrho, r, one), r);
-}
-
-__device__ __forceinline__ F4 vrecip_neg(F4 nrho, F2 one)
-{
-    const F4 r = {f2(rcp_approx(-f2_lo(nrho.a)), rcp_approx(-f2_hi(nrho.a))),
-                  f2(rcp_approx(-f2_lo(nrho.b)), rcp_approx(-f2_hi(nrho.b)))};
-    const F4 e = {vfma(nrho.a, r.a, one), vfma(nrho.b, r.b, one)};
-    return vfma(r, e, r);
-}
-
-// The constants of collide_v.  Two nodes at a time they are kernel arguments, so that the packed
-// instructions take them from there and need no register pair (nor the moves that fill one) for each.
-template <class V>
-struct CollideConsts {
-    V m1, p1, m15, c45, p3, m3;          // -1, 1, -3/2, 9/2, 3, -3
-    V hi[3], lo[3], mhi[3];              // the weights of the rest, axis and diagonal populations: w = hi + lo, and -hi
-    V r, s, t;                           // relaxation: -1/tau (SRT) or -1/tau_s (two-tau); +-(the P factor)
-};
-__host__ __device__ __forceinline__ void cc_set(float &v, float c) { v = c; }
-__host__ __device__ __forceinline__ void cc_set(F2 &v, float c)
-{
-    union { float f[2]; unsigned long long u; } w = {{c, c}};
-    v.v = w.u;
-}
-template <int KIND, class V>
-__host__ __device__ __forceinline__ CollideConsts<V> collide_consts(const Params<float> &p)
-{
-    CollideConsts<V> k;
-    cc_set(k.m1, -1.0f);
-    cc_set(k.p1, 1.0f);
-    cc_set(k.m15, -1.5f);
-    cc_set(k.c45, 4.5f);
-    cc_set(k.p3, 3.0f);
-    cc_set(k.m3, -3.0f);
-    for (int x = 0; x < 3; ++x) {
-        const double w = wgt<double>(x == 0 ? 0 : x == 1 ? 1 : 5);
-        const float hi = (float)w;
-        cc_set(k.hi[x], hi);
-        cc_set(k.lo[x], (float)(w - (double)hi));
-        cc_set(k.mhi[x], -hi);
-    }
-    const float f = KIND == SMRT_COLLISION_SMRT ? p.a4 : p.trt4;
-    cc_set(k.r, KIND == SMRT_COLLISION_SRT ? -p.omega : -p.omega_s);
-    cc_set(k.s, f);
-    cc_set(k.t, -f);
-    return k;
-}
-
-template <bool SPLIT>
-__device__ __forceinline__ float vfma_last(int, float a, float b, float c) { return vfma(a, b, c); }
-template <bool SPLIT>
-__device__ __forceinline__ F2 vfma_last(int dir, F2 a, F2 b, F2 c)
-{
-    if (SPLIT && ex(dir) != 0)
-        return f2(__fmaf_rn(f2_lo(a), f2_lo(b), f2_lo(c)), __fmaf_rn(f2_hi(a), f2_hi(b), f2_hi(c)));
-    return vfma(a, b, c);
-}
-
-template <bool SPLIT>
-__device__ __forceinline__ F4 vfma_last(int dir, F2 a, F4 b, F4 c)
-{
-    return {vfma_last<SPLIT>(dir, a, b.a, c.a), vfma_last<SPLIT>(dir, a, b.b, c.b)};
-}
-template <class V> struct ConstOf { using type = V; };
-template <> struct ConstOf<F4> { using type = F2; };
-
-// The same collision on V = float or F2, every operation rounded as written.  Returns -rho.
-// EXACT: the weight products are those of WeightMul<float, true>; otherwise they are plain, and fused
-// with the operation that follows.  SPLIT: the last operation of the populations that move along x works
-// on each half by itself: its caller regroups the halves for the shift, and a scalar result lands in
-// either half of a register pair without a move.
-template <int KIND, bool EXACT, bool SPLIT, class V>
-__device__ __forceinline__ V collide_v(const CollideConsts<typename ConstOf<V>::type> &k, V g[9])
-{
-    const V drho = vadd(vadd(vadd(vadd(g[0], g[1]), vadd(g[2], g[3])),
-                             vadd(vadd(g[4], g[5]), vadd(g[6], g[7]))), g[8]);
-    const V nrho = vsub(k.m1, drho);
-    const V jx = vadd(vadd(vsub(g[1], g[3]), vsub(g[5], g[6])), vsub(g[8], g[7]));
-    const V jy = vsub(vadd(vsub(g[2], g[4]), vadd(g[5], g[6])), vadd(g[7], g[8]));
-    const V inv = vrecip_neg(nrho, k.p1);
-    const V ux = vmul(jx, inv), uy = vmul(jy, inv);
-    const V base = vfma(k.m15, vfma(jx, ux, vmul(jy, uy)), drho);
-    const V jp = vadd(jx, jy), jm = vsub(jx, jy);
-    const V up = vadd(ux, uy), um = vsub(ux, uy);
-    const V axx = vfma(vmul(k.c45, jx), ux, base), ayy = vfma(vmul(k.c45, jy), uy, base);
-    const V app = vfma(vmul(k.c45, jp), up, base), amm = vfma(vmul(k.c45, jm), um, base);
-    // q_a = w_a x_a
-    const V x[9] = {base, vfma(k.p3, jx, axx), vfma(k.p3, jy, ayy), vfma(k.m3, jx, axx), vfma(k.m3, jy, ayy),
-                    vfma(k.p3, jp, app), vfma(k.m3, jm, amm), vfma(k.m3, jp, app), vfma(k.p3, jm, amm)};
-    V q[9], n[9];
-    #pragma unroll
-    for (int a = 0; a < 9; ++a) {
-        const int w = a == 0 ? 0 : a < 5 ? 1 : 2;
-        if (EXACT) {
-            q[a] = vfma(k.hi[w], x[a], vmul(k.lo[w], x[a]));
-            n[a] = vsub(g[a], q[a]);
-        } else {
-            n[a] = vfma(k.mhi[w], x[a], g[a]);
-        }
-    }
-    if (KIND == SMRT_COLLISION_SRT) {
-        #pragma unroll
-        for (int a = 0; a < 9; ++a) g[a] = vfma_last<SPLIT>(a, k.r, n[a], g[a]);
-        return nrho;
-    }
-    const V pxx = vsub(vadd(n[1], n[3]), vadd(n[2], n[4]));
-    const V pxy = vsub(vadd(n[5], n[7]), vadd(n[6], n[8]));
-    if (KIND == SMRT_COLLISION_SMRT) {
-        if (EXACT) {
-            g[0] = q[0];
-            #pragma unroll
-            for (int a = 1; a < 9; ++a) g[a] = vfma_last<SPLIT>(a, (a & 1) ? k.s : k.t, a < 5 ? pxx : pxy, q[a]);
-        } else {
-            const V txx = vmul(k.s, pxx), txy = vmul(k.s, pxy), sxx = vmul(k.t, pxx), sxy = vmul(k.t, pxy);
-            g[0] = vmul(k.hi[0], x[0]);
-            #pragma unroll
-            for (int a = 1; a < 9; ++a)
-                g[a] = vfma_last<SPLIT>(a, k.hi[a < 5 ? 1 : 2], x[a],
-                                        a < 5 ? ((a & 1) ? txx : sxx) : ((a & 1) ? txy : sxy));
-        }
-    } else {
-        g[0] = vfma(k.r, n[0], g[0]);
-        #pragma unroll
-        for (int a = 1; a < 9; ++a) g[a] = vfma_last<SPLIT>(a, (a & 1) ? k.s : k.t, a < 5 ? pxx : pxy, vfma(k.r, n[a], g[a]));
-    }
-    return nrho;
-}
-
-template <int KIND, bool EXACT = true>
-__device__ __forceinline__ bool collide(const Params<float> &p, float g[9])
-{
-    const float nrho = collide_v<KIND, EXACT, false, float>(collide_consts<KIND, float>(p), g);
-    return nrho < 0.0f && nrho > -INFINITY;
 }
 
 } // namespace smrt

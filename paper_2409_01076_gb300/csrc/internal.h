@@ -45,6 +45,14 @@ struct Scratch {
 constexpr int kResidualSums = 5;        // |du|^2, |u1|^2, rho, rho ux, rho uy
 constexpr int kResidualMaxBlocks = 1216; // 8 x 152 SMs
 
+// Several updates of a small lattice in one launch (tile.cuh).
+struct TilePlan {
+    int W, H, T;         // own nodes of a block, updates per launch
+    int tiles_x, tiles_y;
+    int threads;
+    size_t shared;       // bytes
+};
+
 // Launchers of one storage precision.  `mode` is MODE_AB / MODE_AA_EVEN /
 // MODE_AA_ODD; `kind` an smrt_collision.  Field buffers (double) cover rows
 // [row0, row0 + rows) with row-major [plane][rows][nx] layout.
@@ -53,6 +61,8 @@ struct KernelTable {
                         cudaStream_t s);
     // 2 or 3 updates in one launch, two-buffer layout, nx >= 8 and ny >= 8 (null: not for this precision)
     cudaError_t (*sweep)(int kind, int updates, const void *src, void *dst, const HostParams &p, cudaStream_t s);
+    // t.T updates in one launch, two-buffer layout, nx >= t.T and ny >= t.T
+    cudaError_t (*tile)(int kind, const TilePlan &t, const void *src, void *dst, const HostParams &p, cudaStream_t s);
     cudaError_t (*get_f)(int mode, const void *state, double *f, int row0, int rows,
                          const HostParams &p, cudaStream_t s);
     cudaError_t (*set_f)(int mode, void *state, const double *f, int row0, int rows,

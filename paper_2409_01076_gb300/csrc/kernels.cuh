@@ -17,6 +17,7 @@
 
 #include "d2q9.cuh"
 #include "sweep.cuh"
+#include "tile.cuh"
 
 namespace smrt {
 
@@ -489,19 +490,17 @@ __global__ void init_macros_kernel(typename Prec<PREC>::R *state, const double *
     }
 }
 
-// Moments of Eq. (fea-0) accumulated in double from the canonical offsets.
+// Moments of Eq. (fea-0) in double from the canonical offsets: 28 double operations.  1/rho by recip_d; one
+// correction step makes u the rounded quotient again.
 __device__ __forceinline__ void moments_d(const double g[9], double &rho, double &ux, double &uy)
 {
-    double drho = 0.0, jx = 0.0, jy = 0.0;
-    #pragma unroll
-    for (int a = 0; a < 9; ++a) {
-        drho += g[a];
-        jx += ex(a) * g[a];
-        jy += ey(a) * g[a];
-    }
+    const double drho = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
+    const double d57 = g[5] - g[7], d68 = g[6] - g[8];
+    const double jx = (g[1] - g[3]) + (d57 - d68), jy = (g[2] - g[4]) + (d57 + d68);
     rho = 1.0 + drho;
-    ux = jx / rho;
-    uy = jy / rho;
+    const double inv = recip_d(rho), qx = jx * inv, qy = jy * inv;
+    ux = fma(fma(-qx, rho, jx), inv, qx);
+    uy = fma(fma(-qy, rho, jy), inv, qy);
 }
 
 // s + c += x without rounding error in s + c (Knuth's two-sum; c collects the error terms).
@@ -819,7 +818,7 @@ static __global__ void __launch_bounds__(256) reduce_partials_kernel(const doubl
 // Nodes per thread (VEC: one 16-byte vector or less per population row) and
 // threads per block of the step kernel; overridable at build time for sweeps.
 #ifndef SMRT_VEC_F64
-#define SMRT_VEC_F64 2
+#define SMRT_VEC_F64 1
 #endif
 #ifndef SMRT_VEC_F32
 #define SMRT_VEC_F32 4
@@ -830,11 +829,17 @@ static __global__ void __launch_bounds__(256) reduce_partials_kernel(const doubl
 #ifndef SMRT_BX
 #define SMRT_BX 128
 #endif
+#ifndef SMRT_BX64
+// Double: one node per thread.  The double pipe is the bound (a large lattice takes the same time with one or
+// two), and half as long a chain per warp spreads a small one over the chip: 64^2 8.2 -> 6.2 us per update,
+// 256^2 12.3 -> 10.3, 384^2 26.7 -> 18.5; SRT at 4096^2 1.95 -> 1.81 ms.
+#define SMRT_BX64 64
+#endif
 #ifndef SMRT_BX16
 #define SMRT_BX16 64     // 16-bit storage: measured +1.4 % (AB) / +2.7 % (AA) over 128 at 8192^2
 #endif
 template <int PREC> struct Tune;
-template <> struct Tune<SMRT_PREC_F64> { static constexpr int VEC = SMRT_VEC_F64, BX = SMRT_BX; };
+template <> struct Tune<SMRT_PREC_F64> { static constexpr int VEC = SMRT_VEC_F64, BX = SMRT_BX64; };
 template <> struct Tune<SMRT_PREC_F32> { static constexpr int VEC = SMRT_VEC_F32, BX = SMRT_BX; };
 template <> struct Tune<SMRT_PREC_F16> { static constexpr int VEC = SMRT_VEC_F16, BX = SMRT_BX16; };
 template <> struct Tune<SMRT_PREC_BF16> { static constexpr int VEC = SMRT_VEC_F16, BX = SMRT_BX16; };
@@ -885,47 +890,26 @@ cudaError_t launch_step(int kind, int mode, const void *src, void *dst, const Ho
     }
 }
 
-// T updates in one pass (sweep.cuh).  Rows per segment: the rows that two segments share are computed
-// twice, so long segments do less work, but a lattice that gives each of the 608 SM sub-partitions few
-// warps is bound by the latency of one warp's walk.  Measured (f32, T = 3, 64^2 to 8192^2): a row of one
-// update takes a warp max(0.685, 0.35 + 0.30 w) us with w warps per sub-partition, w also standing for
-// the waves beyond the 4 resident; the minimum of (rows + T - 1) x that is within 4 % of the best of a
-// sweep over rows at every size.  (64^2: 1 row, 6.2 us per single update -> 4.1; 1024^2: 6, 12.3 -> 10.9;
-// 4096^2: 20, 178 -> 88; 8192^2: 64, 694 -> 290.)
-inline int sweep_rows(int strips, int ny, int T)
-{
-    int best = 1;
-    double least = 1e300;
-    for (int rows = 1; rows <= 64 && rows <= ny; ++rows) {
-        const double w = (double)strips * ((ny + rows - 1) / rows) / 608.0;
-        const double one = 0.35 + 0.30 * w;
-        const double cost = (rows + T - 1) * (one > 0.685 ? one : 0.685);
-        if (cost < least) {
-            least = cost;
-            best = rows;
-        }
-    }
-    return best;
-}
-
+// T updates in one pass (sweep.cuh).
 template <int PREC, int KIND, int T>
 cudaError_t launch_sweep_kt(const void *src, void *dst, const HostParams &hp, cudaStream_t s)
 {
     using P = Prec<PREC>;
     using R = typename P::R;
     const Params<typename P::C> p = make_params<typename P::C>(hp);
-    const CollideConsts<F2> cc = collide_consts<KIND, F2>(p);
+    const CollideConsts cc = collide_consts<KIND>(p);
     SweepSalts<T> salt;
     for (int m = 0; m < T; ++m) salt.s[m] = sr_salt(hp.t + m);
-    const int strips = (hp.nx + kSwOwn - 1) / kSwOwn, rows = sweep_rows(strips, hp.ny, T);
+    const int strips = sweep_strips(hp.nx, p.periodic_x), rows = sweep_rows(&strips, &hp.ny, 1, T);
     const unsigned nb = (unsigned)((long long)strips * ((hp.ny + rows - 1) / rows));
+    const bool seam = p.periodic_x && hp.nx % 4 != 0;
+    const size_t smem = sizeof(SweepShared<R, T>) + (seam ? 9 * 32 * sizeof(Raw4<R>) : 0);
+    auto kernel = seam ? sweep_kernel<PREC, KIND, false, T, true> : sweep_kernel<PREC, KIND, false, T, false>;
     if constexpr (PREC == SMRT_PREC_F16 || PREC == SMRT_PREC_BF16) {
-        if (hp.rounding == SMRT_ROUND_STOCHASTIC) {
-            sweep_kernel<PREC, KIND, true, T><<<nb, 32, 0, s>>>((const R *)src, (R *)dst, p, cc, salt, strips, rows);
-            return cudaGetLastError();
-        }
+        if (hp.rounding == SMRT_ROUND_STOCHASTIC)
+            kernel = seam ? sweep_kernel<PREC, KIND, true, T, true> : sweep_kernel<PREC, KIND, true, T, false>;
     }
-    sweep_kernel<PREC, KIND, false, T><<<nb, 32, 0, s>>>((const R *)src, (R *)dst, p, cc, salt, strips, rows);
+    kernel<<<nb, 32, smem, s>>>((const R *)src, (R *)dst, p, cc, salt, strips, rows);
     return cudaGetLastError();
 }
 
@@ -946,6 +930,39 @@ cudaError_t launch_sweep(int kind, int updates, const void *src, void *dst, cons
     case SMRT_COLLISION_SMRT: return launch_sweep_k<PREC, SMRT_COLLISION_SMRT>(updates, src, dst, hp, s);
     case SMRT_COLLISION_SRT: return launch_sweep_k<PREC, SMRT_COLLISION_SRT>(updates, src, dst, hp, s);
     case SMRT_COLLISION_TWO_TAU: return launch_sweep_k<PREC, SMRT_COLLISION_TWO_TAU>(updates, src, dst, hp, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+// Several updates of a small lattice in one launch (tile.cuh).
+template <int PREC, int KIND>
+cudaError_t launch_tile_k(const TilePlan &t, const void *src, void *dst, const HostParams &hp, cudaStream_t s)
+{
+    using P = Prec<PREC>;
+    using R = typename P::R;
+    const Params<typename P::C> p = make_params<typename P::C>(hp);
+    TileSalts salt;
+    for (int m = 0; m < kTileMaxT; ++m) salt.s[m] = sr_salt(hp.t + m);
+    const unsigned nb = (unsigned)(t.tiles_x * t.tiles_y);
+    if constexpr (PREC == SMRT_PREC_F16 || PREC == SMRT_PREC_BF16) {
+        if (hp.rounding == SMRT_ROUND_STOCHASTIC) {
+            tile_kernel<PREC, KIND, true><<<nb, t.threads, t.shared, s>>>((const R *)src, (R *)dst, p, salt, t.W, t.H, t.T,
+                                                                         t.tiles_x);
+            return cudaGetLastError();
+        }
+    }
+    tile_kernel<PREC, KIND, false><<<nb, t.threads, t.shared, s>>>((const R *)src, (R *)dst, p, salt, t.W, t.H, t.T,
+                                                                  t.tiles_x);
+    return cudaGetLastError();
+}
+
+template <int PREC>
+cudaError_t launch_tile(int kind, const TilePlan &t, const void *src, void *dst, const HostParams &hp, cudaStream_t s)
+{
+    switch (kind) {
+    case SMRT_COLLISION_SMRT: return launch_tile_k<PREC, SMRT_COLLISION_SMRT>(t, src, dst, hp, s);
+    case SMRT_COLLISION_SRT: return launch_tile_k<PREC, SMRT_COLLISION_SRT>(t, src, dst, hp, s);
+    case SMRT_COLLISION_TWO_TAU: return launch_tile_k<PREC, SMRT_COLLISION_TWO_TAU>(t, src, dst, hp, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -1059,6 +1076,7 @@ KernelTable make_table()
     t.step = &launch_step<PREC>;
     if constexpr (PREC != SMRT_PREC_F64) t.sweep = &launch_sweep<PREC>;
     else t.sweep = nullptr;
+    t.tile = &launch_tile<PREC>;
     t.get_f = &launch_get_f<PREC>;
     t.set_f = &launch_set_f<PREC>;
     t.init_macros = &launch_init_macros<PREC>;

@@ -22,8 +22,9 @@
 
 namespace smrt {
 
-constexpr int kSwOwn = 120;          // own columns of a strip
-constexpr int kSwBlocks = 16;        // resident per SM: 128 registers
+constexpr int kSwOwn = 120;          // own columns of a strip; the first and last between walls own their outer 4 too
+constexpr int kSwBlocks = 15;        // resident per SM (f32, T = 3: 15 KB of shared memory, 136 registers)
+constexpr int kSwSeamBlocks = 12;    // 168 registers for the element picking at the seam
 constexpr int kSwHalo = 4;           // shared columns on either side: T <= 4, and 16-byte vectors stay aligned
 
 // Four neighbouring stored values, as in memory.
@@ -46,6 +47,13 @@ template <> struct alignas(16) Raw4<float> {
         x = f2_lo(a); y = f2_hi(a); z = f2_lo(b); w = f2_hi(b);
     }
     __device__ __forceinline__ float at(int k) const { return k == 0 ? x : k == 1 ? y : k == 2 ? z : w; }
+    __device__ __forceinline__ void put(int k, float v)
+    {
+        if (k == 0) x = v;
+        if (k == 1) y = v;
+        if (k == 2) z = v;
+        if (k == 3) w = v;
+    }
     __device__ __forceinline__ void zero() { x = y = z = w = 0.0f; }
 };
 template <> struct alignas(8) Raw4<unsigned short> {
@@ -86,6 +94,11 @@ template <> struct alignas(8) Raw4<unsigned short> {
     }
     template <int PREC> __device__ __forceinline__ void round(F2 a, F2 b) { x = narrow<PREC>(a); y = narrow<PREC>(b); }
     __device__ __forceinline__ unsigned short at(int k) const { return (unsigned short)((k < 2 ? x : y) >> (16 * (k & 1))); }
+    __device__ __forceinline__ void put(int k, unsigned short v)
+    {
+        unsigned &h = k < 2 ? x : y;
+        h = (k & 1) ? (h & 0xffffu) | ((unsigned)v << 16) : (h & 0xffff0000u) | v;
+    }
     __device__ __forceinline__ void zero() { x = y = 0u; }
 };
 
@@ -95,15 +108,18 @@ struct SweepSalts {
 };
 
 // A warp's shared memory.  Every lane reads only what it wrote itself, so no barrier is needed.
+//   seam   (behind the struct, only with a periodic x axis and nx % 4 != 0) the second vectors of `row`
 //   row    the raw populations that the next row pulls, copied there while the current row collides
 //   here   between update m and m + 1: of the row that update m collided last, what stays in the row
 //          (0; 1 from c - 1; 3 from c + 1)
 //   below  of that row and of the one before it, what goes up (2; 5 from c - 1; 6 from c + 1)
+//   wall   of that row, f* of the x-wall nodes (3 7 6 of the left one, 1 8 5 of the right one)
 template <class R, int T>
 struct SweepShared {
     Raw4<R> row[9][32];
     Raw4<R> here[T - 1][3][32];
     Raw4<R> below[T - 1][2][3][32];
+    R wall[T - 1][3][2];
 };
 
 template <class R>
@@ -114,46 +130,83 @@ __device__ __forceinline__ void copy_row4(Raw4<R> *smem, const R *gmem)
     else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(gmem) : "memory");
 }
 
-template <class R>
-__device__ __forceinline__ void copy_1(R *smem, const R *gmem)     // 4-byte elements only
-{
-    const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gmem) : "memory");
-}
-
 template <bool B>
 struct Bool {
     static constexpr bool value = B;
 };
 
+// Strips that cover nx columns.
+inline int sweep_strips(int nx, bool periodic_x)
+{
+    return periodic_x ? (nx + kSwOwn - 1) / kSwOwn : (nx <= 128 ? 1 : (nx - 2 * kSwHalo + kSwOwn - 1) / kSwOwn);
+}
+
+// Rows per segment of `count` lattices swept together.  The rows that two segments share are computed
+// twice, so long segments do less work, but few warps per SM sub-partition (608 of them) are bound by the
+// latency of one warp's walk.  Measured (f32, T = 3, 64^2 to 8192^2): a row of one update takes a warp
+// max(0.685, 0.35 + 0.30 w) us with w warps per sub-partition, w also standing for the waves beyond the 4
+// resident; the minimum of (rows + T - 1) x that is within 4 % of the best of a sweep over rows at every
+// size.  (1024^2: 6 rows, 12.3 us per single update -> 10.9; 4096^2: 20, 178 -> 88; 8192^2: 64, 694 -> 290.)
+inline int sweep_rows(const int *strips, const int *ny, int count, int T)
+{
+    int best = 1;
+    double least = 1e300;
+    for (int rows = 1; rows <= 64; ++rows) {
+        double items = 0.0;
+        for (int k = 0; k < count; ++k) items += (double)strips[k] * ((ny[k] + rows - 1) / rows);
+        const double one = 0.35 + 0.30 * items / 608.0;
+        const double cost = (rows + T - 1) * (one > 0.685 ? one : 0.685);
+        if (cost < least) {
+            least = cost;
+            best = rows;
+        }
+    }
+    return best;
+}
+
 // T updates of the rows [r0, r1) of one strip, by one warp (blockDim.x == 32).  Needs nx >= 8 and
 // ny >= 8.  salt.s[m] is the stochastic-rounding salt of update m.
-template <int PREC, int KIND, bool SR, int T>
+// SEAM: a periodic x axis with nx % 4 != 0.
+template <int PREC, int KIND, bool SR, int T, bool SEAM>
 __device__ __forceinline__ void sweep(const typename Prec<PREC>::R *__restrict__ src,
                                       typename Prec<PREC>::R *__restrict__ dst,
-                                      const Params<typename Prec<PREC>::C> &p, const CollideConsts<F2> &cc,
+                                      const Params<typename Prec<PREC>::C> &p, const CollideConsts &cc,
                                       const SweepSalts<T> &salt, int strip, int r0, int r1,
-                                      SweepShared<typename Prec<PREC>::R, T> &sm)
+                                      SweepShared<typename Prec<PREC>::R, T> &sm,
+                                      Raw4<typename Prec<PREC>::R> *seam)
 {
     static_assert(T >= 2 && T <= kSwHalo, "shared columns");
     using P = Prec<PREC>;
     using R = typename P::R;
     using Row = Raw4<R>;
     const int lane = threadIdx.x;
-    const int x0 = strip * kSwOwn, c4 = x0 - kSwHalo + 4 * lane;     // the lane's first column, may lie outside
     const bool wall_x = !p.periodic_x, wall_y = !p.periodic_y;
+    const int x0 = strip * kSwOwn - (wall_x ? 0 : kSwHalo);          // the warp's first column, and the lane's:
+    const int c4 = x0 + 4 * lane;                                    // either may lie outside
+    const bool own = (lane >= 1 || (wall_x && x0 == 0)) && (lane <= kSwOwn / 4 || (wall_x && x0 + 128 >= p.nx)) &&
+                     c4 < p.nx;
     const int ny = p.ny;
 
-    // Column to load from, and whether the four columns are one aligned vector there.  Behind a wall
-    // the values are not used (any stored column will do); on a periodic axis the columns wrap.
-    int lc = max(0, min(c4, p.pitch - 4));
-    bool vec = true;
+    // Column to load from.  Behind a wall the values are not used (any stored column will do); on a
+    // periodic axis the columns wrap.  A lane whose four columns are not one aligned vector there (nx not
+    // a multiple of 4, by the seam) loads the two vectors that hold them, at lc and lw, and picks its
+    // elements when it reads: n1 of them from the first, behind its first `o`, then the second's.
+    int lc = max(0, min(c4, p.pitch - 4)), lw = 0, n1 = 4, o = 0;
     if (!wall_x) {
         lc = c4 < 0 ? c4 + p.nx : c4 % p.nx;
-        vec = (lc & 3) == 0 && lc + 4 <= p.nx;
+        o = SEAM ? lc & 3 : 0;
+        if (SEAM && o != 0) {
+            lc -= o;
+            lw = min(lc + 4, p.pitch - 4);
+            n1 = 4 - o;
+        } else if (SEAM && lc + 4 > p.nx) {
+            n1 = p.nx - lc;
+        }
     }
+    const bool vec = !SEAM || n1 == 4;
+    const bool all_vec = !SEAM || __all_sync(0xffffffffu, vec);
     // x-wall nodes: at most one per lane (nx >= 8)
-    const bool edge_strip = wall_x && (x0 == 0 || x0 + kSwOwn + kSwHalo >= p.nx);
+    const bool edge_strip = wall_x && (x0 == 0 || x0 + 128 >= p.nx);
     const bool at_left = wall_x && c4 == 0, at_right = wall_x && c4 < p.nx && c4 + 4 >= p.nx;
     const int kx = at_right ? (p.nx - 1) & 3 : 0;                    // that node's place in its lane
     const R *col = src + lc;
@@ -171,18 +224,8 @@ __device__ __forceinline__ void sweep(const typename Prec<PREC>::R *__restrict__
         for (int a = 0; a < 9; ++a) {
             const R *q = (ey(a) == 0 ? mid : ey(a) > 0 ? (b ? mid : below) : (t ? mid : above)) +
                          (size_t)((ey(a) > 0 && b) || (ey(a) < 0 && t) ? opp(a) : a) * (size_t)p.plane;
-            if (vec) {
-                copy_row4<R>(&sm.row[a][lane], q);
-            } else if (sizeof(R) == 4) {
-                #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    copy_1<R>(reinterpret_cast<R *>(&sm.row[a][lane]) + k, q + (lc + k >= p.nx ? k - p.nx : k));
-            } else {
-                R e[4];
-                #pragma unroll
-                for (int k = 0; k < 4; ++k) e[k] = q[lc + k >= p.nx ? k - p.nx : k];
-                sm.row[a][lane].set(e);
-            }
+            copy_row4<R>(&sm.row[a][lane], q);
+            if (!vec) copy_row4<R>(&seam[a * 32 + lane], q + (lw - lc));
         }
     };
     unsigned worst[4] = {0u, 0u, 0u, 0u};                            // of -rho by column, in an order that ends with the diverged ones
@@ -223,7 +266,7 @@ __device__ __forceinline__ void sweep(const typename Prec<PREC>::R *__restrict__
         F4 v[9];
         #pragma unroll
         for (int a = 0; a < 9; ++a) v[a] = {g[0][a], g[1][a]};
-        const F4 nr = collide_v<KIND, P::kExactWeights, !decltype(last)::value && sizeof(R) == 4, F4>(cc, v);
+        const F4 nr = collide_v<KIND, P::kExactWeights, !decltype(last)::value && sizeof(R) == 4>(cc, v);
         #pragma unroll
         for (int a = 0; a < 9; ++a) { g[0][a] = v[a].a; g[1][a] = v[a].b; }
         #pragma unroll
@@ -254,13 +297,6 @@ __device__ __forceinline__ void sweep(const typename Prec<PREC>::R *__restrict__
         }
     };
 
-    // f* of the x-wall node of the row that update m collided last (3 7 6 at the left wall, 1 8 5 at the right)
-    R el[T - 1][3];
-    #pragma unroll
-    for (int m = 0; m < T - 1; ++m)
-        #pragma unroll
-        for (int x = 0; x < 3; ++x) el[m][x] = 0;
-
     // update m collides the rows [r0 - (T - 1 - m), r1 + (T - 1 - m)) that the lattice has
     const int first = wall_y ? max(r0 - (T - 1), 0) : r0 - (T - 1);
     const int last = r1 + T - 2;                                     // with T - 1 rows of lag: row r1 - 1 stored
@@ -275,6 +311,14 @@ __device__ __forceinline__ void sweep(const typename Prec<PREC>::R *__restrict__
             #pragma unroll
             for (int a = 0; a < 9; ++a) {
                 f[a] = sm.row[a][lane];
+                if (!all_vec) {
+                    const R *x = reinterpret_cast<const R *>(&sm.row[a][lane]) + o;
+                    const R *y = reinterpret_cast<const R *>(&seam[a * 32 + lane]) - n1;
+                    R v[4];
+                    #pragma unroll
+                    for (int k = 0; k < 4; ++k) v[k] = (k < n1 ? x : y)[k];
+                    f[a].set(v);
+                }
                 if (ex(a) != 0 && !((ey(a) > 0 && b) || (ey(a) < 0 && t))) f[a] = ex(a) > 0 ? f[a].up() : f[a].down();
             }
             R e[3] = {0, 0, 0};                                      // f*_{abar} of the x-wall node
@@ -296,6 +340,12 @@ __device__ __forceinline__ void sweep(const typename Prec<PREC>::R *__restrict__
             const int par = (j + 1) & 1;
             Row (&here)[3][32] = sm.here[m - 1];
             Row (&below)[2][3][32] = sm.below[m - 1];
+            R (&wall)[3][2] = sm.wall[m - 1];
+            R e[3] = {0, 0, 0};                                      // of row j
+            if (edge_strip && (at_left || at_right)) {
+                #pragma unroll
+                for (int x = 0; x < 3; ++x) e[x] = wall[x][at_right];
+            }
             Row g[9];
             if (node_row) {
                 g[4] = f[4];
@@ -305,10 +355,11 @@ __device__ __forceinline__ void sweep(const typename Prec<PREC>::R *__restrict__
                 g[4] = below[par ^ 1][0][lane];
                 g[7] = below[par ^ 1][1][lane].down();
                 g[8] = below[par ^ 1][2][lane].up();
+                if (at_left) g[8].put(0, e[2]);                      // (shifted out at the outermost lanes)
+                if (at_right) g[7].put(kx, e[2]);
             }
             g[0] = here[0][lane]; g[1] = here[1][lane]; g[3] = here[2][lane];
             g[2] = below[par][0][lane]; g[5] = below[par][1][lane]; g[6] = below[par][2][lane];
-            const R e[3] = {el[m - 1][0], el[m - 1][1], el[m - 1][2]};
             if (node_row) {
                 // row j + 1 takes the place of row j
                 if (at_floor(j + 1)) {                               // below row 0: its own 4, 7, 8 come back
@@ -322,14 +373,10 @@ __device__ __forceinline__ void sweep(const typename Prec<PREC>::R *__restrict__
                 here[0][lane] = f[0];
                 here[1][lane] = f[1].up();
                 here[2][lane] = f[3].down();
-                if (edge_strip) {
-                    #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (kx == k) {
-                            el[m - 1][0] = at_right ? f[1].at(k) : f[3].at(k);
-                            el[m - 1][1] = at_right ? f[8].at(k) : f[7].at(k);
-                            el[m - 1][2] = at_right ? f[5].at(k) : f[6].at(k);
-                        }
+                if (edge_strip && (at_left || at_right)) {
+                    wall[0][at_right] = at_right ? f[1].at(kx) : f[3].at(0);
+                    wall[1][at_right] = at_right ? f[8].at(kx) : f[7].at(0);
+                    wall[2][at_right] = at_right ? f[5].at(kx) : f[6].at(0);
                 }
             }
             if (!wanted) break;
@@ -339,7 +386,7 @@ __device__ __forceinline__ void sweep(const typename Prec<PREC>::R *__restrict__
                 for (int a = 0; a < 9; ++a) f[a] = g[a];
             } else {
                 collide_row(Bool<true>(), g, e, j, salt.s[m]);
-                if (lane >= 1 && lane <= kSwOwn / 4 && c4 < p.nx) {
+                if (own) {
                     R *q = dst + (size_t)j * (size_t)p.pitch + c4;   // past nx: the row's padding
                     #pragma unroll
                     for (int a = 0; a < 9; ++a) g[a].store(q + (size_t)a * (size_t)p.plane);
@@ -351,21 +398,24 @@ __device__ __forceinline__ void sweep(const typename Prec<PREC>::R *__restrict__
     bool bad = false;
     #pragma unroll
     for (int k = 0; k < 4; ++k) bad = bad || (worst[k] >= 0x7f7fffffu && c4 + k < p.nx);
-    if (bad && lane >= 1 && lane <= kSwOwn / 4) atomicOr(p.flag, 1);
+    if (bad && own) atomicOr(p.flag, 1);
 }
 
 // One item (segment, strip) per block, strips fastest: concurrent blocks share the rows between their
 // segments and the columns between their strips in L2.
-template <int PREC, int KIND, bool SR, int T>
-__global__ void __launch_bounds__(32, kSwBlocks)
+template <int PREC, int KIND, bool SR, int T, bool SEAM>
+__global__ void __launch_bounds__(32, SEAM ? kSwSeamBlocks : kSwBlocks)
 sweep_kernel(const typename Prec<PREC>::R *src, typename Prec<PREC>::R *dst,
-             const Params<typename Prec<PREC>::C> p, const CollideConsts<F2> cc, const SweepSalts<T> salt, int strips,
+             const Params<typename Prec<PREC>::C> p, const CollideConsts cc, const SweepSalts<T> salt, int strips,
              int rows)
 {
-    __shared__ __align__(16) SweepShared<typename Prec<PREC>::R, T> sm;
+    extern __shared__ __align__(16) unsigned char sweep_smem[];
+    using Shared = SweepShared<typename Prec<PREC>::R, T>;
+    Shared &sm = *reinterpret_cast<Shared *>(sweep_smem);
+    Raw4<typename Prec<PREC>::R> *seam = reinterpret_cast<Raw4<typename Prec<PREC>::R> *>(sweep_smem + sizeof(Shared));
     const int seg = blockIdx.x / strips, strip = blockIdx.x - seg * strips;
     const int r0 = seg * rows;
-    sweep<PREC, KIND, SR, T>(src, dst, p, cc, salt, strip, r0, min(r0 + rows, p.ny), sm);
+    sweep<PREC, KIND, SR, T, SEAM>(src, dst, p, cc, salt, strip, r0, min(r0 + rows, p.ny), sm, seam);
 }
 
 } // namespace smrt
