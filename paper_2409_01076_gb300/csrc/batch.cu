@@ -109,6 +109,69 @@ batch_step_kernel(const typename Prec<PREC>::R *src, typename Prec<PREC>::R *dst
     }
 }
 
+// ---- several updates per pass (sweep.cuh) ----------------------------------------------
+// One block per (lattice, segment, strip); the same bits as single updates.
+struct BatchSweep {
+    Params<float> p;
+    F2 r, s, t;          // the lattice's own relaxation (CollideConsts)
+    long long offset;
+    int strips, rows;
+};
+
+// The grid is the item list's length when the launch was made or captured; items of lattices that have
+// retired since are gone from the list, whose length is read from device memory.
+template <int KIND, int T, bool SEAM>
+__global__ void __launch_bounds__(32, SEAM ? kSwSeamBlocks : kSwBlocks)
+batch_sweep_kernel(const float *src, float *dst, const BatchSweep *__restrict__ sw, const int2 *__restrict__ items,
+                   const int *__restrict__ counts, const CollideConsts cc)
+{
+    extern __shared__ __align__(16) unsigned char sweep_smem[];
+    __shared__ __align__(16) unsigned long long rec[sizeof(BatchSweep) / 8];
+    using Shared = SweepShared<float, T>;
+    Shared &sm = *reinterpret_cast<Shared *>(sweep_smem);
+    Raw4<float> *seam = reinterpret_cast<Raw4<float> *>(sweep_smem + sizeof(Shared));
+    if ((int)blockIdx.x >= counts[3]) return;
+    const int2 w = items[blockIdx.x];
+    const unsigned long long *g = reinterpret_cast<const unsigned long long *>(sw + w.x);
+    for (int k = threadIdx.x; k < (int)(sizeof(BatchSweep) / 8); k += 32) rec[k] = g[k];
+    __syncwarp();
+    const BatchSweep &L = *reinterpret_cast<const BatchSweep *>(rec);
+    CollideConsts k = cc;
+    k.r = L.r;
+    k.s = L.s;
+    k.t = L.t;
+    const int strips = L.strips, rows = L.rows, seg = w.y / strips, r0 = seg * rows;
+    SweepSalts<T> salt = {};
+    sweep<SMRT_PREC_F32, KIND, false, T, SEAM>(src + L.offset, dst + L.offset, L.p, k, salt, w.y - seg * strips, r0,
+                                               min(r0 + rows, L.p.ny), sm, seam);
+}
+
+template <int KIND, int T>
+cudaError_t launch_batch_sweep_kt(const float *src, float *dst, const void *sw, const int2 *items, const int *counts,
+                                  int n, bool seam, cudaStream_t s)
+{
+    HostParams hp = {};
+    hp.tau = hp.tau_s = 1.0;
+    const CollideConsts cc = collide_consts<KIND>(make_params<float>(hp));
+    const size_t smem = sizeof(SweepShared<float, T>) + (seam ? 9 * 32 * sizeof(Raw4<float>) : 0);
+    auto kernel = seam ? batch_sweep_kernel<KIND, T, true> : batch_sweep_kernel<KIND, T, false>;
+    kernel<<<n, 32, smem, s>>>(src, dst, (const BatchSweep *)sw, items, counts, cc);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_batch_sweep(int kind, int updates, const void *src, void *dst, const void *sw, const int2 *items,
+                               const int *counts, int n, bool seam, cudaStream_t s)
+{
+    const float *a = (const float *)src;
+    float *b = (float *)dst;
+    if (n < 1) return cudaSuccess;
+    if (kind == SMRT_COLLISION_SMRT)
+        return updates == 3 ? launch_batch_sweep_kt<SMRT_COLLISION_SMRT, 3>(a, b, sw, items, counts, n, seam, s)
+                            : launch_batch_sweep_kt<SMRT_COLLISION_SMRT, 2>(a, b, sw, items, counts, n, seam, s);
+    return updates == 3 ? launch_batch_sweep_kt<SMRT_COLLISION_SRT, 3>(a, b, sw, items, counts, n, seam, s)
+                        : launch_batch_sweep_kt<SMRT_COLLISION_SRT, 2>(a, b, sw, items, counts, n, seam, s);
+}
+
 // Per-lattice residual pass over u(t) = moments of the canonical f(t): stores u(t)
 // as u_prev; with `accumulate` it first sums |u(t) - u_prev|^2, |u(t)|^2 and rho(t)
 // over the lattice's nodes.  One 256-node row segment per tile.
@@ -441,6 +504,12 @@ struct smrt_batch_t {
     double2 *d_uprev = nullptr;
     double *d_partials = nullptr, *d_sums = nullptr, *h_sums = nullptr;
     long long max_tiles = 0, max_work = 0;
+    // sweeps (F32, two-buffer, every lattice at least 8 x 8; else sweep_rows == 0)
+    int sweep_rows = 0, sweep_items = 0;   // rows per segment; items of the active lattices
+    bool sweep_seam = false;
+    void *d_sweep = nullptr;
+    int2 *d_items = nullptr;
+    long long max_items = 0;
     cudaGraphExec_t graph = nullptr;
     int graph_k = 0, graph_mode = -1, graph_shape = -1, graph_kind = -1;
     bool list_dirty = true;
@@ -505,7 +574,11 @@ int upload_lists(smrt_batch_t *b)
     const size_t cb = b->prec == SMRT_PREC_F64 ? smrt::cav_bytes<SMRT_PREC_F64>() : smrt::cav_bytes<SMRT_PREC_F32>();
     b->h_cav.resize(cb * b->count);
     std::vector<int> act, rpre(1, 0);
-    std::vector<int2> work, rwork;
+    std::vector<int2> work, rwork, items;
+    std::vector<smrt::BatchSweep> sweeps(b->sweep_rows ? b->count : 0);
+    work.reserve(b->max_work);
+    rwork.reserve(b->max_tiles);
+    items.reserve(b->max_items);
     for (int k = 0; k < b->count; ++k) {
         const Lat &L = b->lat[k];
         HostParams hp = lat_params(b, k);
@@ -520,8 +593,24 @@ int upload_lists(smrt_batch_t *b)
             nb = smrt::step_blocks<SMRT_PREC_F32>(b->shape, g);
             smrt::fill_cav<SMRT_PREC_F32>(&b->h_cav[cb * k], hp, g, L.offset, L.uoff);
         }
+        int strips = 0, segs = 0;
+        if (b->sweep_rows) {
+            smrt::BatchSweep &w = sweeps[k];
+            w.p = smrt::make_params<float>(hp);
+            const smrt::CollideConsts cc = b->collision == SMRT_COLLISION_SMRT
+                                               ? smrt::collide_consts<SMRT_COLLISION_SMRT>(w.p)
+                                               : smrt::collide_consts<SMRT_COLLISION_SRT>(w.p);
+            w.r = cc.r;
+            w.s = cc.s;
+            w.t = cc.t;
+            w.offset = L.offset;
+            w.strips = strips = smrt::sweep_strips(L.nx, w.p.periodic_x);
+            w.rows = b->sweep_rows;
+            segs = (L.ny + w.rows - 1) / w.rows;
+        }
         if (L.state != ST_ACTIVE) continue;
         act.push_back(k);
+        for (int j = 0; j < strips * segs; ++j) items.push_back(make_int2(k, j));
         for (int j = 0; j < nb; ++j) work.push_back(make_int2(k, j));
         const int tiles = L.ny * ((L.nx + smrt::kResTile - 1) / smrt::kResTile);
         for (int j = 0; j < tiles; ++j) rwork.push_back(make_int2(k, j));
@@ -529,7 +618,9 @@ int upload_lists(smrt_batch_t *b)
     }
     if ((long long)work.size() > b->max_work || (long long)rwork.size() > b->max_tiles)
         return bfail(b, SMRT_ERR_STATE, "work list exceeds its allocation");
-    int counts[3] = {(int)act.size(), (int)work.size(), rpre.back()};
+    if ((long long)items.size() > b->max_items) return bfail(b, SMRT_ERR_STATE, "item list exceeds its allocation");
+    b->sweep_items = (int)items.size();
+    int counts[4] = {(int)act.size(), (int)work.size(), rpre.back(), b->sweep_items};
     BTRY(b, cudaMemcpyAsync(b->d_cav, b->h_cav.data(), b->h_cav.size(), cudaMemcpyHostToDevice, b->stream));
     if (!act.empty()) {
         BTRY(b, cudaMemcpyAsync(b->d_act, act.data(), act.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream));
@@ -538,6 +629,12 @@ int upload_lists(smrt_batch_t *b)
         BTRY(b, cudaMemcpyAsync(b->d_rwork, rwork.data(), rwork.size() * sizeof(int2), cudaMemcpyHostToDevice,
                                 b->stream));
     }
+    if (b->sweep_rows)
+        BTRY(b, cudaMemcpyAsync(b->d_sweep, sweeps.data(), sweeps.size() * sizeof(sweeps[0]), cudaMemcpyHostToDevice,
+                                b->stream));
+    if (!items.empty())
+        BTRY(b, cudaMemcpyAsync(b->d_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice,
+                                b->stream));
     BTRY(b, cudaMemcpyAsync(b->d_counts, counts, sizeof(counts), cudaMemcpyHostToDevice, b->stream));
     // the host arrays are stack/vector temporaries: wait until the copies have read them
     BTRY(b, cudaStreamSynchronize(b->stream));
@@ -570,6 +667,28 @@ cudaError_t enqueue_step(smrt_batch_t *b, long long t)
                                                      b->d_counts, b->sms, b->stream);
     return smrt::launch_batch_step<SMRT_PREC_F32>(b->collision, mode, b->shape, src, dst, b->d_cav, b->d_work,
                                                  b->d_counts, b->sms, b->stream);
+}
+
+// Enqueue the updates t .. t + n - 1, in passes of up to three where the batch sweeps.  parity >= 0: in a
+// number of passes of that parity (n >= 1, and n even for parity 0), so that the caller knows the buffer the
+// state ends in.  b->cur follows the passes.
+cudaError_t enqueue_steps(smrt_batch_t *b, long long t, long long n, int parity)
+{
+    cudaError_t e = cudaSuccess;
+    long long passes = b->sweep_rows ? (n + 2) / 3 : n;
+    if (parity >= 0 && passes % 2 != parity) ++passes;
+    while (e == cudaSuccess && n > 0) {
+        const int k = (int)((n + passes - 1) / passes);       // at most 3, larger ones first
+        if (k == 1) e = enqueue_step(b, t);
+        else
+            e = smrt::launch_batch_sweep(b->collision, k, b->buf[b->cur], b->buf[1 - b->cur], b->d_sweep, b->d_items,
+                                         b->d_counts, b->sweep_items, b->sweep_seam, b->stream);
+        if (e == cudaSuccess && b->layout == SMRT_LAYOUT_AB) b->cur = 1 - b->cur;
+        t += k;
+        n -= k;
+        --passes;
+    }
+    return e;
 }
 
 cudaError_t enqueue_residual(smrt_batch_t *b, long long t, int cur, int accumulate)
@@ -676,7 +795,23 @@ int smrt_batch_create(int count, const int *nx, const int *ny, const double *tau
                                                                                          layout == SMRT_LAYOUT_AB));
         if (w > b->max_work) b->max_work = w;
     }
-    if (b->max_work >= (1LL << 31)) {
+    if (precision == SMRT_PREC_F32 && layout == SMRT_LAYOUT_AB) {
+        const bool periodic_x = (bc_flags & 3u) == SMRT_BC_PERIODIC;
+        std::vector<int> strips, rows;
+        bool fits = true;
+        for (const Lat &L : b->lat) {
+            fits = fits && L.nx >= 8 && L.ny >= 8;
+            b->sweep_seam = b->sweep_seam || (periodic_x && L.nx % 4 != 0);
+            strips.push_back(smrt::sweep_strips(L.nx, periodic_x));
+            rows.push_back(L.ny);
+        }
+        if (fits) {
+            b->sweep_rows = smrt::sweep_rows(strips.data(), rows.data(), count, 3);
+            for (int k = 0; k < count; ++k)
+                b->max_items += (long long)strips[k] * ((rows[k] + b->sweep_rows - 1) / b->sweep_rows);
+        }
+    }
+    if (b->max_work >= (1LL << 31) || b->max_items >= (1LL << 31)) {
         delete b;
         return bfail(nullptr, SMRT_ERR_ARG, "smrt_batch_create: batch too large");
     }
@@ -690,8 +825,10 @@ int smrt_batch_create(int count, const int *nx, const int *ny, const double *tau
     if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_act, sizeof(int) * count);
     if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_rpre, sizeof(int) * (count + 1));
     if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_work, sizeof(int2) * (size_t)b->max_work);
+    if (e == cudaSuccess && b->sweep_rows) e = cudaMalloc(&b->d_sweep, sizeof(smrt::BatchSweep) * (size_t)count);
+    if (e == cudaSuccess && b->sweep_rows) e = cudaMalloc((void **)&b->d_items, sizeof(int2) * (size_t)b->max_items);
     if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_rwork, sizeof(int2) * (size_t)tiles);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_counts, sizeof(int) * 3);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_counts, sizeof(int) * 4);
     if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_flags, sizeof(int) * count);
     if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_uprev, sizeof(double2) * (size_t)uoff);
     if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_partials, sizeof(double) * 3 * (size_t)tiles);
@@ -753,12 +890,8 @@ int smrt_batch_step(smrt_batch_t *b, long long n)
         int rc = upload_lists(b);
         if (rc != SMRT_OK) return rc;
     }
-    long long t = active_t(b);
-    for (long long s = 0; s < n; ++s, ++t) {
-        cudaError_t e = enqueue_step(b, t);
-        if (e != cudaSuccess) return bfail(b, SMRT_ERR_CUDA, "batch step launch: %s", cudaGetErrorString(e));
-        if (b->layout == SMRT_LAYOUT_AB) b->cur = 1 - b->cur;
-    }
+    const cudaError_t e = enqueue_steps(b, active_t(b), n, -1);
+    if (e != cudaSuccess) return bfail(b, SMRT_ERR_CUDA, "batch step launch: %s", cudaGetErrorString(e));
     for (Lat &L : b->lat)
         if (L.state == ST_ACTIVE) {
             L.t += n;
@@ -867,10 +1000,15 @@ int smrt_batch_run(smrt_batch_t *b, double tol, long long check_every, long long
         int cur0 = b->cur;
         // one-step: check_every - 1 updates, snapshot u, one more update, compare;
         // stride: check_every updates, compare with the previous check's snapshot
-        for (long long s = 0; e == cudaSuccess && s < check_every; ++s) {
-            if (!stride && s == check_every - 1) e = enqueue_residual(b, t + s, b->cur, 0);
-            if (e == cudaSuccess) e = enqueue_step(b, t + s);
-            if (b->layout == SMRT_LAYOUT_AB) b->cur = 1 - b->cur;
+        // (an even number of passes in all: the state ends in the buffer it started from)
+        if (e == cudaSuccess) {
+            if (stride) {
+                e = enqueue_steps(b, t, check_every, 0);
+            } else {
+                e = enqueue_steps(b, t, check_every - 1, 1);
+                if (e == cudaSuccess) e = enqueue_residual(b, t + check_every - 1, b->cur, 0);
+                if (e == cudaSuccess) e = enqueue_steps(b, t + check_every - 1, 1, 1);
+            }
         }
         if (e == cudaSuccess) e = enqueue_residual(b, t + check_every, b->cur, 1);
         if (e == cudaSuccess)
@@ -897,7 +1035,7 @@ int smrt_batch_run(smrt_batch_t *b, double tol, long long check_every, long long
     while (active_count(b) > 0) {
         BTRY(b, cudaGraphLaunch(b->graph, b->stream));
         BTRY(b, cudaStreamSynchronize(b->stream));
-        // check_every is even, so the AB buffer holding the state is unchanged
+        // an even number of passes: the AB buffer holding the state is unchanged
         bool changed = false;
         for (int k = 0; k < b->count; ++k) {
             Lat &L = b->lat[k];
@@ -1014,7 +1152,7 @@ void smrt_batch_destroy(smrt_batch_t *b)
     for (int k = 0; k < 2; ++k)
         if (b->buf[k]) cudaFree(b->buf[k]);
     void *dev[] = {b->d_cav, b->d_act, b->d_rpre, b->d_work, b->d_rwork, b->d_counts, b->d_flags, b->d_uprev,
-                   b->d_partials, b->d_sums};
+                   b->d_partials, b->d_sums, b->d_sweep, b->d_items};
     for (void *p : dev)
         if (p) cudaFree(p);
     if (b->h_sums) cudaFreeHost(b->h_sums);
