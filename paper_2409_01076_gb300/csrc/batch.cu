@@ -14,6 +14,7 @@
 
 #include <math.h>
 #include <stdarg.h>
+#include <stdint.h>
 #include <stdio.h>
 
 #include <new>
@@ -505,11 +506,14 @@ struct smrt_batch_t {
     double *d_partials = nullptr, *d_sums = nullptr, *h_sums = nullptr;
     long long max_tiles = 0, max_work = 0;
     // sweeps (F32, two-buffer, every lattice at least 8 x 8; else sweep_rows == 0)
+    int h_counts[4] = {0, 0, 0, 0};
     int sweep_rows = 0, sweep_items = 0;   // rows per segment; items of the active lattices
     bool sweep_seam = false;
     void *d_sweep = nullptr;
     int2 *d_items = nullptr;
     long long max_items = 0;
+    double *d_stage = nullptr;
+    size_t stage_doubles = 0;
     cudaGraphExec_t graph = nullptr;
     int graph_k = 0, graph_mode = -1, graph_shape = -1, graph_kind = -1;
     bool list_dirty = true;
@@ -568,17 +572,20 @@ int nshapes(int prec)
     return prec == SMRT_PREC_F64 ? smrt::Shapes<SMRT_PREC_F64>::n : smrt::Shapes<SMRT_PREC_F32>::n;
 }
 
-// Rebuild descriptors (for the current tile shape) and the work lists of the active lattices.
-int upload_lists(smrt_batch_t *b)
+// Rebuild descriptors (for the current tile shape) and the work lists of the active lattices.  shape_only: the
+// active lattices are those of the last call, and only what depends on the tile shape is rebuilt.
+int upload_lists(smrt_batch_t *b, bool shape_only = false)
 {
     const size_t cb = b->prec == SMRT_PREC_F64 ? smrt::cav_bytes<SMRT_PREC_F64>() : smrt::cav_bytes<SMRT_PREC_F32>();
     b->h_cav.resize(cb * b->count);
     std::vector<int> act, rpre(1, 0);
     std::vector<int2> work, rwork, items;
-    std::vector<smrt::BatchSweep> sweeps(b->sweep_rows ? b->count : 0);
+    std::vector<smrt::BatchSweep> sweeps(b->sweep_rows && !shape_only ? b->count : 0);
     work.reserve(b->max_work);
-    rwork.reserve(b->max_tiles);
-    items.reserve(b->max_items);
+    if (!shape_only) {
+        rwork.reserve(b->max_tiles);
+        items.reserve(b->max_items);
+    }
     for (int k = 0; k < b->count; ++k) {
         const Lat &L = b->lat[k];
         HostParams hp = lat_params(b, k);
@@ -594,7 +601,7 @@ int upload_lists(smrt_batch_t *b)
             smrt::fill_cav<SMRT_PREC_F32>(&b->h_cav[cb * k], hp, g, L.offset, L.uoff);
         }
         int strips = 0, segs = 0;
-        if (b->sweep_rows) {
+        if (!sweeps.empty()) {
             smrt::BatchSweep &w = sweeps[k];
             w.p = smrt::make_params<float>(hp);
             const smrt::CollideConsts cc = b->collision == SMRT_COLLISION_SMRT
@@ -609,36 +616,39 @@ int upload_lists(smrt_batch_t *b)
             segs = (L.ny + w.rows - 1) / w.rows;
         }
         if (L.state != ST_ACTIVE) continue;
+        for (int j = 0; j < nb; ++j) work.push_back(make_int2(k, j));
+        if (shape_only) continue;
         act.push_back(k);
         for (int j = 0; j < strips * segs; ++j) items.push_back(make_int2(k, j));
-        for (int j = 0; j < nb; ++j) work.push_back(make_int2(k, j));
         const int tiles = L.ny * ((L.nx + smrt::kResTile - 1) / smrt::kResTile);
         for (int j = 0; j < tiles; ++j) rwork.push_back(make_int2(k, j));
         rpre.push_back(rpre.back() + tiles);
     }
-    if ((long long)work.size() > b->max_work || (long long)rwork.size() > b->max_tiles)
+    if ((long long)work.size() > b->max_work || (long long)rwork.size() > b->max_tiles ||
+        (long long)items.size() > b->max_items)
         return bfail(b, SMRT_ERR_STATE, "work list exceeds its allocation");
-    if ((long long)items.size() > b->max_items) return bfail(b, SMRT_ERR_STATE, "item list exceeds its allocation");
-    b->sweep_items = (int)items.size();
-    int counts[4] = {(int)act.size(), (int)work.size(), rpre.back(), b->sweep_items};
-    BTRY(b, cudaMemcpyAsync(b->d_cav, b->h_cav.data(), b->h_cav.size(), cudaMemcpyHostToDevice, b->stream));
-    if (!act.empty()) {
-        BTRY(b, cudaMemcpyAsync(b->d_act, act.data(), act.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream));
-        BTRY(b, cudaMemcpyAsync(b->d_rpre, rpre.data(), rpre.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream));
-        BTRY(b, cudaMemcpyAsync(b->d_work, work.data(), work.size() * sizeof(int2), cudaMemcpyHostToDevice, b->stream));
-        BTRY(b, cudaMemcpyAsync(b->d_rwork, rwork.data(), rwork.size() * sizeof(int2), cudaMemcpyHostToDevice,
-                                b->stream));
+    b->h_counts[1] = (int)work.size();
+    if (!shape_only) {
+        b->h_counts[0] = (int)act.size();
+        b->h_counts[2] = rpre.back();
+        b->h_counts[3] = b->sweep_items = (int)items.size();
     }
-    if (b->sweep_rows)
-        BTRY(b, cudaMemcpyAsync(b->d_sweep, sweeps.data(), sweeps.size() * sizeof(sweeps[0]), cudaMemcpyHostToDevice,
-                                b->stream));
-    if (!items.empty())
-        BTRY(b, cudaMemcpyAsync(b->d_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice,
-                                b->stream));
-    BTRY(b, cudaMemcpyAsync(b->d_counts, counts, sizeof(counts), cudaMemcpyHostToDevice, b->stream));
-    // the host arrays are stack/vector temporaries: wait until the copies have read them
+    auto copy = [&](void *dst, const void *src, size_t bytes) {
+        return bytes ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, b->stream) : cudaSuccess;
+    };
+    BTRY(b, copy(b->d_cav, b->h_cav.data(), b->h_cav.size()));
+    BTRY(b, copy(b->d_work, work.data(), work.size() * sizeof(int2)));
+    if (!shape_only) {
+        BTRY(b, copy(b->d_act, act.data(), act.size() * sizeof(int)));
+        BTRY(b, copy(b->d_rpre, rpre.data(), rpre.size() * sizeof(int)));
+        BTRY(b, copy(b->d_rwork, rwork.data(), rwork.size() * sizeof(int2)));
+        BTRY(b, copy(b->d_sweep, sweeps.data(), sweeps.size() * sizeof(smrt::BatchSweep)));
+        BTRY(b, copy(b->d_items, items.data(), items.size() * sizeof(int2)));
+    }
+    BTRY(b, copy(b->d_counts, b->h_counts, sizeof(b->h_counts)));
+    // the host arrays are temporaries: wait until the copies have read them
     BTRY(b, cudaStreamSynchronize(b->stream));
-    b->list_dirty = false;
+    if (!shape_only) b->list_dirty = false;
     return SMRT_OK;
 }
 
@@ -715,6 +725,31 @@ void* lattice_state(smrt_batch_t *b, int k)
 {
     const void *base = b->buf[b->layout == SMRT_LAYOUT_AB ? b->lat[k].cur : 0];
     return (char *)base + (size_t)b->lat[k].offset * b->elem;
+}
+
+// Memory the kernels may read and write in place: device memory of the batch's device, 8-byte aligned.
+bool device_memory(const smrt_batch_t *b, const void *p)
+{
+    cudaPointerAttributes at;
+    const cudaError_t e = cudaPointerGetAttributes(&at, p);
+    cudaGetLastError();
+    return e == cudaSuccess && (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) &&
+           at.device == b->device && ((uintptr_t)p & 7u) == 0;
+}
+
+// At least n doubles of device scratch for fields in other memory, kept until the batch is destroyed (the
+// largest lattice's at most).  Every call that uses it waits for its stream before it returns.
+int ensure_stage(smrt_batch_t *b, size_t n, double **out)
+{
+    if (b->stage_doubles < n) {
+        if (b->d_stage) cudaFree(b->d_stage);
+        b->d_stage = nullptr;
+        b->stage_doubles = 0;
+        BTRY(b, cudaMalloc((void **)&b->d_stage, sizeof(double) * n));
+        b->stage_doubles = n;
+    }
+    *out = b->d_stage;
+    return SMRT_OK;
 }
 
 int check_index(smrt_batch_t *b, int k)
@@ -913,6 +948,10 @@ int smrt_batch_autotune(smrt_batch_t *b, int steps, int *choice)
     if (steps < 2) return bfail(b, SMRT_ERR_ARG, "smrt_batch_autotune: steps must be >= 2");
     steps += steps % 2;                 // AB: leave the state in its buffer
     drop_graph(b);
+    if (b->list_dirty) {
+        const int rc = upload_lists(b);
+        if (rc != SMRT_OK) return rc;
+    }
     // time each candidate on a scratch copy of the state so the lattices do not advance
     const int nbuf = b->layout == SMRT_LAYOUT_AB ? 2 : 1;
     void *save = nullptr;
@@ -928,7 +967,7 @@ int smrt_batch_autotune(smrt_batch_t *b, int steps, int *choice)
     const long long t0 = active_t(b);
     for (int sh = 0; e == cudaSuccess && sh < nshapes(b->prec); ++sh) {
         b->shape = sh;
-        int rc = upload_lists(b);
+        int rc = upload_lists(b, true);
         if (rc != SMRT_OK) { e = cudaErrorUnknown; break; }
         long long t = t0;
         e = enqueue_step(b, t);              // warm-up launch
@@ -962,7 +1001,7 @@ int smrt_batch_autotune(smrt_batch_t *b, int steps, int *choice)
     // the divergence words may have been set by a candidate run on the copy: clear them
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_flags, 0, sizeof(int) * b->count, b->stream);
     b->shape = best_shape;
-    int rc = upload_lists(b);
+    int rc = upload_lists(b, true);
     if (e != cudaSuccess) return bfail(b, SMRT_ERR_CUDA, "smrt_batch_autotune: %s", cudaGetErrorString(e));
     if (rc != SMRT_OK) return rc;
     if (choice) *choice = best_shape;
@@ -1073,19 +1112,15 @@ int smrt_batch_get_f(smrt_batch_t *b, int k, double *f)
     int rc = check_index(b, k);
     if (rc != SMRT_OK) return rc;
     if (!f) return bfail(b, SMRT_ERR_ARG, "smrt_batch_get_f: f is NULL");
-    cudaPointerAttributes at;
-    cudaError_t e = cudaPointerGetAttributes(&at, f);
-    cudaGetLastError();
-    const bool dev = e == cudaSuccess && (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged);
     const Lat &L = b->lat[k];
     HostParams hp = lat_params(b, k);
     double *out = f;
-    if (!dev) BTRY(b, cudaMalloc((void **)&out, sizeof(double) * 9 * (size_t)L.nodes));
-    e = table(b->prec).get_f(mode_of(b, L.t), lattice_state(b, k), out, 0, L.ny, hp, b->stream);
+    const bool dev = device_memory(b, f);
+    if (!dev && (rc = ensure_stage(b, 9 * (size_t)L.nodes, &out)) != SMRT_OK) return rc;
+    cudaError_t e = table(b->prec).get_f(mode_of(b, L.t), lattice_state(b, k), out, 0, L.ny, hp, b->stream);
     if (e == cudaSuccess && !dev)
         e = cudaMemcpyAsync(f, out, sizeof(double) * 9 * (size_t)L.nodes, cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    if (!dev) cudaFree(out);
     if (e != cudaSuccess) return bfail(b, SMRT_ERR_CUDA, "smrt_batch_get_f: %s", cudaGetErrorString(e));
     return SMRT_OK;
 }
@@ -1097,16 +1132,20 @@ int smrt_batch_macros(smrt_batch_t *b, int k, double *rho, double *u)
     if (!rho || !u) return bfail(b, SMRT_ERR_ARG, "smrt_batch_macros: rho and u are required");
     const Lat &L = b->lat[k];
     HostParams hp = lat_params(b, k);
-    double *tmp = nullptr;
-    BTRY(b, cudaMalloc((void **)&tmp, sizeof(double) * 3 * (size_t)L.nodes));
-    cudaError_t e = table(b->prec).macros(mode_of(b, L.t), lattice_state(b, k), tmp, tmp + L.nodes, 0, L.ny, hp,
-                                          b->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(rho, tmp, sizeof(double) * (size_t)L.nodes, cudaMemcpyDefault, b->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(u, tmp + L.nodes, sizeof(double) * 2 * (size_t)L.nodes, cudaMemcpyDefault, b->stream);
+    const bool dr = device_memory(b, rho), du = device_memory(b, u);
+    double *tr = rho, *tu = u;
+    if (!dr || !du) {
+        double *tmp = nullptr;
+        if ((rc = ensure_stage(b, 3 * (size_t)L.nodes, &tmp)) != SMRT_OK) return rc;
+        if (!dr) tr = tmp;
+        if (!du) tu = tmp + L.nodes;
+    }
+    cudaError_t e = table(b->prec).macros(mode_of(b, L.t), lattice_state(b, k), tr, tu, 0, L.ny, hp, b->stream);
+    if (e == cudaSuccess && !dr)
+        e = cudaMemcpyAsync(rho, tr, sizeof(double) * (size_t)L.nodes, cudaMemcpyDefault, b->stream);
+    if (e == cudaSuccess && !du)
+        e = cudaMemcpyAsync(u, tu, sizeof(double) * 2 * (size_t)L.nodes, cudaMemcpyDefault, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    cudaFree(tmp);
     if (e != cudaSuccess) return bfail(b, SMRT_ERR_CUDA, "smrt_batch_macros: %s", cudaGetErrorString(e));
     return SMRT_OK;
 }
@@ -1120,16 +1159,25 @@ int smrt_batch_init_macros(smrt_batch_t *b, int k, const double *rho, const doub
     if (L.state != ST_ACTIVE || L.t != active_t(b))
         return bfail(b, SMRT_ERR_STATE, "smrt_batch_init_macros: lattice %d is retired", k);
     HostParams hp = lat_params(b, k);
-    double *tmp = nullptr;
-    BTRY(b, cudaMalloc((void **)&tmp, sizeof(double) * 3 * (size_t)L.nodes));
-    cudaError_t e = cudaMemcpyAsync(tmp, rho, sizeof(double) * (size_t)L.nodes, cudaMemcpyDefault, b->stream);
+    const bool dr = device_memory(b, rho), du = device_memory(b, u);
+    const double *sr = rho, *su = u;
+    cudaError_t e = cudaSuccess;
+    if (!dr || !du) {
+        double *tmp = nullptr;
+        if ((rc = ensure_stage(b, 3 * (size_t)L.nodes, &tmp)) != SMRT_OK) return rc;
+        if (!dr) {
+            sr = tmp;
+            e = cudaMemcpyAsync(tmp, rho, sizeof(double) * (size_t)L.nodes, cudaMemcpyDefault, b->stream);
+        }
+        if (!du) {
+            su = tmp + L.nodes;
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(tmp + L.nodes, u, sizeof(double) * 2 * (size_t)L.nodes, cudaMemcpyDefault, b->stream);
+        }
+    }
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(tmp + L.nodes, u, sizeof(double) * 2 * (size_t)L.nodes, cudaMemcpyDefault, b->stream);
-    if (e == cudaSuccess)
-        e = table(b->prec).init_macros(mode_of(b, L.t), lattice_state(b, k), tmp, tmp + L.nodes, 0, L.ny, hp,
-                                       b->stream);
+        e = table(b->prec).init_macros(mode_of(b, L.t), lattice_state(b, k), sr, su, 0, L.ny, hp, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    cudaFree(tmp);
     if (e != cudaSuccess) return bfail(b, SMRT_ERR_CUDA, "smrt_batch_init_macros: %s", cudaGetErrorString(e));
     return SMRT_OK;
 }
@@ -1152,7 +1200,7 @@ void smrt_batch_destroy(smrt_batch_t *b)
     for (int k = 0; k < 2; ++k)
         if (b->buf[k]) cudaFree(b->buf[k]);
     void *dev[] = {b->d_cav, b->d_act, b->d_rpre, b->d_work, b->d_rwork, b->d_counts, b->d_flags, b->d_uprev,
-                   b->d_partials, b->d_sums, b->d_sweep, b->d_items};
+                   b->d_partials, b->d_sums, b->d_sweep, b->d_items, b->d_stage};
     for (void *p : dev)
         if (p) cudaFree(p);
     if (b->h_sums) cudaFreeHost(b->h_sums);
