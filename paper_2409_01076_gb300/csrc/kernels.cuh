@@ -398,6 +398,25 @@ __device__ __forceinline__ void pull_canonical(const typename Prec<PREC>::R *sta
     }
 }
 
+// Where f_a of a node whose nine source nodes lie inside the lattice (no wall, no wrap) is stored.
+template <int MODE, class C>
+__device__ __forceinline__ size_t inner_at(const Params<C> &p, int a, int i, int j)
+{
+    const long long node = (long long)j * p.pitch + i;
+    if (MODE == MODE_AA_EVEN) return (size_t)(a * p.plane + node);
+    return (size_t)((MODE == MODE_AB ? a : opp(a)) * p.plane + node - (ey(a) * p.pitch + ex(a)));
+}
+
+// pull_canonical for such a node.
+template <int PREC, int MODE>
+__device__ __forceinline__ void pull_inner(const typename Prec<PREC>::R *state, const Params<typename Prec<PREC>::C> &p,
+                                           int i, int j, typename Prec<PREC>::C g[9])
+{
+    using P = Prec<PREC>;
+    #pragma unroll
+    for (int a = 0; a < 9; ++a) g[a] = P::to_c(state[inner_at<MODE>(p, a, i, j)]);
+}
+
 template <int PREC, int MODE>
 __global__ void get_f_kernel(const typename Prec<PREC>::R *state, double *f, int row0, int rows,
                              const Params<typename Prec<PREC>::C> p)
@@ -436,29 +455,49 @@ __global__ void set_f_kernel(typename Prec<PREC>::R *state, const double *f, int
 // significant bits); the weight product is rounded as for an exact weight.
 template <int PREC, int MODE, int A>
 __device__ __forceinline__ void init_store_f(typename Prec<PREC>::R *state, const Params<float> &p, int i, int j,
-                                             float drho, float d, float ux, float uy, float uu)
+                                             bool inner, float drho, float d, float ux, float uy, float uu)
 {
     using P = Prec<PREC>;
     const float eu = float(ex(A)) * ux + float(ey(A)) * uy;
     float g = WeightMul<float>::template mul<A>(drho + d * (3.0f * eu + 4.5f * eu * eu - 1.5f * uu));
+    if (inner) {
+        state[inner_at<MODE>(p, A, i, j)] = P::to_r(g);
+        return;
+    }
     const Loc L = pull_loc<MODE>(p, A, i, j);
     if (L.side >= 0) g -= p.corr[L.side][A];
     state[at(p.plane, p.pitch, L.plane, L.j, L.i)] = P::to_r(g);
 }
 
+// Blocks of the field kernels below: 256 consecutive nodes of one row, so that a node's row and column
+// need no division per thread.
+constexpr int kFieldBX = 256;
+inline unsigned field_blocks(int rows, int nx)
+{
+    return (unsigned)((long long)rows * ((nx + kFieldBX - 1) / kFieldBX));
+}
+__device__ __forceinline__ bool field_node(int nx, int &r, int &i)
+{
+    const unsigned per_row = (unsigned)(nx + kFieldBX - 1) / kFieldBX;
+    r = (int)(blockIdx.x / per_row);
+    i = (int)((blockIdx.x - (unsigned)r * per_row) * kFieldBX + threadIdx.x);
+    return i < nx;
+}
+
 // f = f^eq(rho, u) (Eq. feq-full), written as offsets through the pull map;
 // rho == NULL selects rho = 1, u = 0.  rho and u may be device memory or host memory
 // the device can address (page-locked and mapped).
+// Double offsets in the form of the double collision (32 operations instead of about 75: 8192^2 9.66 -> 4.39 ms).
 template <int PREC, int MODE>
-__global__ void init_macros_kernel(typename Prec<PREC>::R *state, const double *rho, const double *u,
-                                   int row0, int rows, const Params<typename Prec<PREC>::C> p)
+__global__ void __launch_bounds__(kFieldBX)
+init_macros_kernel(typename Prec<PREC>::R *state, const double *rho, const double *u,
+                   int row0, int rows, const Params<typename Prec<PREC>::C> p)
 {
     using P = Prec<PREC>;
-    long long n = (long long)rows * p.nx;
-    long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    int r = (int)(t / p.nx), i = (int)(t % p.nx), j = row0 + r;
-    size_t q = (size_t)r * p.nx + i;
+    int r, i;
+    if (!field_node(p.nx, r, i)) return;
+    const int j = row0 + r;
+    const size_t q = (size_t)r * p.nx + i;
     double d = 1.0, ux = 0.0, uy = 0.0;           // rho == NULL: the resting state
     if (rho) {
         d = rho[q];
@@ -466,27 +505,35 @@ __global__ void init_macros_kernel(typename Prec<PREC>::R *state, const double *
         uy = u[(size_t)rows * p.nx + q];
     }
     if constexpr (PREC == SMRT_PREC_F64) {
-        double uu = ux * ux + uy * uy;
+        const double drho = d - 1.0, jx = d * ux, jy = d * uy;
+        const double xx = jx * ux, yy = jy * uy, xy = jx * uy;
+        const double K = xx + yy, k12 = K * (1.0 / 12.0), n = 0.25 * (xx - yy), m = 0.25 * xy;
+        const double a0 = fma(drho, 1.0 / 9.0, k12), b0 = fma(drho, 1.0 / 36.0, k12);
+        const double ax = a0 + n, ay = a0 - n, bp = b0 + m, bm = b0 - m, jp = jx + jy, jm = jx - jy;
+        const double g[9] = {fma(drho, 4.0 / 9.0, K * (-2.0 / 3.0)),
+                             fma(jx, 1.0 / 3.0, ax), fma(jy, 1.0 / 3.0, ay), fma(jx, -1.0 / 3.0, ax),
+                             fma(jy, -1.0 / 3.0, ay), fma(jp, 1.0 / 12.0, bp), fma(jm, -1.0 / 12.0, bm),
+                             fma(jp, -1.0 / 12.0, bp), fma(jm, 1.0 / 12.0, bm)};
         #pragma unroll
         for (int a = 0; a < 9; ++a) {
-            double eu = ex(a) * ux + ey(a) * uy;
-            double g = wgt<double>(a) * ((d - 1.0) + d * (3.0 * eu + 4.5 * eu * eu - 1.5 * uu));
-            Loc L = pull_loc<MODE>(p, a, i, j);
-            if (L.side >= 0) g -= (double)p.corr[L.side][a];
-            state[at(p.plane, p.pitch, L.plane, L.j, L.i)] = P::to_r((typename P::C)g);
+            const Loc L = pull_loc<MODE>(p, a, i, j);
+            double v = g[a];
+            if (L.side >= 0) v -= (double)p.corr[L.side][a];
+            state[at(p.plane, p.pitch, L.plane, L.j, L.i)] = P::to_r((typename P::C)v);
         }
     } else {
         const float drho = (float)(d - 1.0), df = (float)d, fx = (float)ux, fy = (float)uy;
         const float uu = fx * fx + fy * fy;
-        init_store_f<PREC, MODE, 0>(state, p, i, j, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 1>(state, p, i, j, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 2>(state, p, i, j, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 3>(state, p, i, j, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 4>(state, p, i, j, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 5>(state, p, i, j, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 6>(state, p, i, j, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 7>(state, p, i, j, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 8>(state, p, i, j, drho, df, fx, fy, uu);
+        const bool inner = i >= 1 && i + 1 < p.nx && j >= 1 && j + 1 < p.ny;
+        init_store_f<PREC, MODE, 0>(state, p, i, j, inner, drho, df, fx, fy, uu);
+        init_store_f<PREC, MODE, 1>(state, p, i, j, inner, drho, df, fx, fy, uu);
+        init_store_f<PREC, MODE, 2>(state, p, i, j, inner, drho, df, fx, fy, uu);
+        init_store_f<PREC, MODE, 3>(state, p, i, j, inner, drho, df, fx, fy, uu);
+        init_store_f<PREC, MODE, 4>(state, p, i, j, inner, drho, df, fx, fy, uu);
+        init_store_f<PREC, MODE, 5>(state, p, i, j, inner, drho, df, fx, fy, uu);
+        init_store_f<PREC, MODE, 6>(state, p, i, j, inner, drho, df, fx, fy, uu);
+        init_store_f<PREC, MODE, 7>(state, p, i, j, inner, drho, df, fx, fy, uu);
+        init_store_f<PREC, MODE, 8>(state, p, i, j, inner, drho, df, fx, fy, uu);
     }
 }
 
@@ -512,11 +559,26 @@ __device__ __forceinline__ void two_sum_acc(float &s, float &c, float x)
     s = t;
 }
 
-// The moments of Eq. (fea-0) of nine float offsets, in double, with few double operations:
-// each sum is formed in float as an unevaluated pair hi + lo (two-sum), which carries about
-// 48 significant bits of it, and 1 / rho is the float reciprocal refined by two Newton steps
-// (to double rounding).  The double pipe is the scarce unit of this GPU; this form needs about
-// a quarter of the double operations of moments_d, whose results it matches to ~1e-14.
+// x as a double by integer operations (a conversion costs this GPU as much as a double operation): sign and
+// mantissa shifted into place, the exponent rebiased.  Not for the x that wide_special names.
+__device__ __forceinline__ double wide_d(float x)
+{
+    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+    const unsigned hi = m == 0u ? 0u : (b & 0x80000000u) | ((m >> 3) + 0x38000000u);
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
+// Subnormals, infinities and NaN.
+__device__ __forceinline__ bool wide_special(float x)
+{
+    const unsigned m = __float_as_uint(x) & 0x7fffffffu;
+    return m - 1u < 0x007fffffu || m >= 0x7f800000u;
+}
+
+// The moments of Eq. (fea-0) of nine float offsets, in double, with nine double operations: each sum is formed
+// in float as an unevaluated pair hi + lo (two-sum), which carries about 48 significant bits of it, and 1 / rho is
+// recip_d.  The double pipe is the scarce unit of this GPU; moments_d takes 28 operations and nine conversions on
+// float offsets, results match it to ~1e-15.  (With the pairs converted by the double pipe and Newton's steps from
+// a converted float reciprocal this took 18: 8192^2 fields 2.25 -> 1.15 ms; their bytes take 0.59.)
 __device__ __forceinline__ void moments_f(const float g[9], double &rho, double &ux, double &uy)
 {
     float s0 = g[0], c0 = 0.0f, sx = g[1], cx = 0.0f, sy = g[2], cy = 0.0f;
@@ -538,12 +600,21 @@ __device__ __forceinline__ void moments_f(const float g[9], double &rho, double 
     two_sum_acc(sy, cy, g[6]);
     two_sum_acc(sy, cy, -g[7]);
     two_sum_acc(sy, cy, -g[8]);
-    rho = 1.0 + ((double)s0 + (double)c0);
-    const double r0 = (double)(1.0f / (float)rho);
-    const double r1 = r0 * (2.0 - rho * r0);
-    const double inv = r1 * (2.0 - rho * r1);
-    ux = ((double)sx + (double)cx) * inv;
-    uy = ((double)sy + (double)cy) * inv;
+    double d0, dx, dy;
+    if (wide_special(s0) || wide_special(c0) || wide_special(sx) || wide_special(cx) || wide_special(sy) ||
+        wide_special(cy)) {
+        d0 = (double)s0 + (double)c0;
+        dx = (double)sx + (double)cx;
+        dy = (double)sy + (double)cy;
+    } else {
+        d0 = wide_d(s0) + wide_d(c0);
+        dx = wide_d(sx) + wide_d(cx);
+        dy = wide_d(sy) + wide_d(cy);
+    }
+    rho = 1.0 + d0;
+    const double inv = recip_d(rho);
+    ux = dx * inv;
+    uy = dy * inv;
 }
 
 // moments_d for double offsets, moments_f for float ones.
@@ -557,18 +628,19 @@ __device__ __forceinline__ void moments_any(const float g[9], double &rho, doubl
 }
 
 template <int PREC, int MODE>
-__global__ void macros_kernel(const typename Prec<PREC>::R *state, double *rho, double *u, int row0,
-                              int rows, const Params<typename Prec<PREC>::C> p)
+__global__ void __launch_bounds__(kFieldBX)
+macros_kernel(const typename Prec<PREC>::R *state, double *rho, double *u, int row0, int rows,
+              const Params<typename Prec<PREC>::C> p)
 {
-    long long n = (long long)rows * p.nx;
-    long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    int r = (int)(t / p.nx), i = (int)(t % p.nx);
+    int r, i;
+    if (!field_node(p.nx, r, i)) return;
+    const int j = row0 + r;
     typename Prec<PREC>::C g[9];
-    pull_canonical<PREC, MODE>(state, p, i, row0 + r, g);
+    if (i >= 1 && i + 1 < p.nx && j >= 1 && j + 1 < p.ny) pull_inner<PREC, MODE>(state, p, i, j, g);
+    else pull_canonical<PREC, MODE>(state, p, i, j, g);
     double rr, ux, uy;
     moments_any(g, rr, ux, uy);
-    size_t q = (size_t)r * p.nx + i;
+    const size_t q = (size_t)r * p.nx + i;
     if (rho) rho[q] = rr;
     if (u) {
         u[q] = ux;
@@ -603,22 +675,6 @@ __device__ __forceinline__ double warp_sum(double v)
     #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
     return v;
-}
-
-// pull_canonical for a node whose nine source nodes lie inside the lattice (no wall, no wrap).
-template <int PREC, int MODE>
-__device__ __forceinline__ void pull_inner(const typename Prec<PREC>::R *state, const Params<typename Prec<PREC>::C> &p,
-                                           int i, int j, typename Prec<PREC>::C g[9])
-{
-    using P = Prec<PREC>;
-    const typename P::R *s0 = state + (size_t)j * (size_t)p.pitch + (size_t)i;
-    #pragma unroll
-    for (int a = 0; a < 9; ++a) {
-        const long long off = (MODE == MODE_AA_EVEN) ? (long long)a * p.plane
-                              : (long long)(MODE == MODE_AB ? a : opp(a)) * p.plane -
-                                    (long long)ey(a) * p.pitch - ex(a);
-        g[a] = P::to_c(s0[off]);
-    }
 }
 
 // f(t) of node (i, j) of the sweep, wrapped onto the lattice; false where (i, j) is behind a wall or
@@ -1012,8 +1068,8 @@ cudaError_t launch_init_macros(int mode, void *state, const double *rho, const d
     using P = Prec<PREC>;
     const Params<typename P::C> p = make_params<typename P::C>(hp);
     if (rows <= 0) return cudaSuccess;
-    const unsigned nb = node_blocks(rows, hp.nx, 256);
-    SMRT_MODE_SWITCH(mode, (init_macros_kernel<PREC, M><<<nb, 256, 0, s>>>((typename P::R *)state, rho, u, row0, rows, p)));
+    const unsigned nb = field_blocks(rows, hp.nx);
+    SMRT_MODE_SWITCH(mode, (init_macros_kernel<PREC, M><<<nb, kFieldBX, 0, s>>>((typename P::R *)state, rho, u, row0, rows, p)));
     return cudaGetLastError();
 }
 
@@ -1024,8 +1080,8 @@ cudaError_t launch_macros(int mode, const void *state, double *rho, double *u, i
     using P = Prec<PREC>;
     const Params<typename P::C> p = make_params<typename P::C>(hp);
     if (rows <= 0) return cudaSuccess;
-    const unsigned nb = node_blocks(rows, hp.nx, 256);
-    SMRT_MODE_SWITCH(mode, (macros_kernel<PREC, M><<<nb, 256, 0, s>>>((const typename P::R *)state, rho, u, row0, rows, p)));
+    const unsigned nb = field_blocks(rows, hp.nx);
+    SMRT_MODE_SWITCH(mode, (macros_kernel<PREC, M><<<nb, kFieldBX, 0, s>>>((const typename P::R *)state, rho, u, row0, rows, p)));
     return cudaGetLastError();
 }
 
