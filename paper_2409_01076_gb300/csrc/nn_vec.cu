@@ -57,7 +57,17 @@ __device__ __forceinline__ size_t blocked_off(int p, int g, int G, int HW)
     return (((size_t)n * G + g) * HW + rem) * 8;
 }
 
-__device__ __forceinline__ float sigm(float z) { return 1.0f / (1.0f + expf(-z)); }
+// 1 / (1 + e^-z), the quotient rounded correctly.  1 + e^-z is at least 1; below 2^125 the hardware's
+// reciprocal, good to one unit in the last place, and one Newton step with its exact residual round like the
+// division (Markstein 1990; compared for every such float), without the division's branch.
+__device__ __forceinline__ float sigm(float z)
+{
+    const float d = 1.0f + expf(-z);
+    if (!(d < 4.0e37f)) return 1.0f / d;
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return fmaf(r, fmaf(-d, r, 1.0f), r);
+}
 
 // z = x + bias; a = SiLU(z) (or z); ab = half(a) blocked (V == 8 only).  Thread: pixel p, group g.
 template <int V>
@@ -87,30 +97,36 @@ __global__ void bias_act_vec(const float *__restrict__ x, const float *__restric
 }
 
 // dz = da * SiLU'(z) (or da); db[c] += sum over pixels of dz; dzb = half(dz) blocked (V == 8 only).
-// The grid stride is a multiple of G = C / V, so every thread keeps one channel group and sums its
-// share of db in registers; a block adds its per-channel sums with one atomic each.
-template <int V>
 // dp (may be NULL): a gradient at half resolution whose 2x2 average-pooling adjoint (0.25 dp of the
 // parent pixel) is added to da first; W is the full-resolution width.
-__global__ void bias_act_bwd_vec(const float *__restrict__ da, const float *__restrict__ z, int P, int C, int act,
+// The grid stride is a multiple of G = C / V, so every thread keeps one channel group, sums its share of
+// db in registers and steps from pixel to pixel without a division; a block adds its per-channel sums
+// with one atomic each.  Reads 8 and writes 2 bytes a value.  The grid is one wave of resident blocks: 16
+// blocks per SM, of which 5 fit, left the last wave nearly empty (16 x 256^2 x 32: 82 -> 59 us, 49 at the copy
+// rate; with dp 97 -> 68; 4, 6 and 8 blocks per SM measured 61 / 75, 62 / 69 and 69 / 76).
+constexpr int kBwdBlocks = 5;
+template <int V>
+__global__ void __launch_bounds__(256, kBwdBlocks)
+bias_act_bwd_vec(const float *__restrict__ da, const float *__restrict__ z, int P, int C, int act,
                                  float *dz, float *db, __half *__restrict__ dzb, int HW,
                                  const float *__restrict__ dp = nullptr, int W = 0)
 {
     extern __shared__ float sdb[];          // C floats
     for (int c = threadIdx.x; c < C; c += blockDim.x) sdb[c] = 0.0f;
     __syncthreads();
-    const int G = C / V, total = P * G;
+    const int G = C / V;
     const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
-    const int g = t0 % G;
+    const int g = t0 % G, step = (int)(gridDim.x * blockDim.x) / G;
     float acc[V];
     #pragma unroll
     for (int i = 0; i < V; ++i) acc[i] = 0.0f;
-    for (int t = t0; t < total; t += gridDim.x * blockDim.x) {
-        const int p = t / G;
+    int p = t0 / G, n = 0, r = p;           // pixel, its image and its place there
+    while (r >= HW && n < P / HW) { r -= HW; ++n; }
+    for (; p < P; p += step) {
         const size_t off = (size_t)p * C + (size_t)g * V;
         Vec<V> d = ldv<V>(da + off);
         if (dp) {
-            const int n = p / HW, r = p - n * HW, yy = r / W, xx = r - yy * W;
+            const int yy = r / W, xx = r - yy * W;
             const Vec<V> q = ldv<V>(dp + (((size_t)n * (HW / W / 2) + yy / 2) * (W / 2) + xx / 2) * C + (size_t)g * V);
             #pragma unroll
             for (int i = 0; i < V; ++i) d.v[i] += 0.25f * q.v[i];
@@ -127,8 +143,10 @@ __global__ void bias_act_bwd_vec(const float *__restrict__ da, const float *__re
         #pragma unroll
         for (int i = 0; i < V; ++i) acc[i] += d.v[i];
         if constexpr (V == 8) {
-            if (dzb) st_half8(dzb + blocked_off(p, g, G, HW), d);
+            if (dzb) st_half8(dzb + (((size_t)n * G + g) * HW + r) * 8, d);
         }
+        r += step;
+        while (r >= HW) { r -= HW; ++n; }
     }
     if (db) {
         #pragma unroll
@@ -224,105 +242,101 @@ __global__ void add_vec(const float *a, const float *b, int n4, float *y)
     }
 }
 
-__device__ __forceinline__ float warp_sum(float v)
-{
-    #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // 1x1 convolution with few outputs (the network's head), float32 on the CUDA cores: a product of
 // COUT x C per pixel is far too narrow for the tensor cores and is bound by reading x.
-// Forward: y[p][o] = sum_c x[p][c] w[o][c] + b[o].  Thread: one pixel.
+// Forward: y[p][o] = sum_c x[p][c] w[o][c] + b[o].  Thread: one pixel, its channels summed in order.  A block
+// stages its 256 pixels in shared memory with coalesced 16-byte loads, 32 channels at a time (a thread that
+// reads its own pixel from memory touches a line of its own with every load: 43 us at 16 x 256^2 x 32, whose
+// bytes take 22; staged: 32 us).
+constexpr int kHeadBX = 256, kHeadC = 32;
 template <int COUT>
-__global__ void conv1x1_small(const float *__restrict__ x, int P, int C, const float *__restrict__ w,
-                              const float *__restrict__ bias, float *__restrict__ y)
+__global__ void __launch_bounds__(kHeadBX)
+conv1x1_small(const float *__restrict__ x, int P, int C, const float *__restrict__ w, const float *__restrict__ bias,
+              float *__restrict__ y)
 {
-    extern __shared__ float sw[];           // COUT x C weights
-    for (int i = threadIdx.x; i < COUT * C; i += blockDim.x) sw[i] = w[i];
-    __syncthreads();
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
+    __shared__ __align__(16) float sx[kHeadBX * (kHeadC + 1)];
+    __shared__ float sw[COUT * 64];
+    for (int i = threadIdx.x; i < COUT * C; i += kHeadBX) sw[i] = w[i];
+    for (unsigned p0 = blockIdx.x * kHeadBX; p0 < (unsigned)P; p0 += gridDim.x * kHeadBX) {
+        const int np = min(kHeadBX, P - (int)p0);
         float acc[COUT];
         #pragma unroll
         for (int o = 0; o < COUT; ++o) acc[o] = bias ? bias[o] : 0.0f;
-        const float *xp = x + (size_t)p * C;
-        for (int c = 0; c < C; c += 4) {
-            const Vec<4> v = ldv<4>(xp + c);
-            #pragma unroll
-            for (int o = 0; o < COUT; ++o)
+        for (int c0 = 0; c0 < C; c0 += kHeadC) {
+            const int nc = min(kHeadC, C - c0), nq = nc / 4;
+            __syncthreads();
+            for (int k = threadIdx.x; k < np * nq; k += kHeadBX) {
+                const int q = k / nq, c = 4 * (k - q * nq);
+                const Vec<4> v = ldv<4>(x + (size_t)(p0 + q) * C + c0 + c);
                 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[o] = fmaf(v.v[i], sw[o * C + c + i], acc[o]);
+                for (int i = 0; i < 4; ++i) sx[q * (kHeadC + 1) + c + i] = v.v[i];
+            }
+            __syncthreads();
+            if ((int)threadIdx.x < np) {
+                for (int c = 0; c < nc; ++c) {
+                    const float v = sx[threadIdx.x * (kHeadC + 1) + c];
+                    #pragma unroll
+                    for (int o = 0; o < COUT; ++o) acc[o] = fmaf(v, sw[o * C + c0 + c], acc[o]);
+                }
+            }
         }
-        #pragma unroll
-        for (int o = 0; o < COUT; ++o) y[(size_t)p * COUT + o] = acc[o];
+        if ((int)threadIdx.x < np) {
+            #pragma unroll
+            for (int o = 0; o < COUT; ++o) y[(size_t)(p0 + threadIdx.x) * COUT + o] = acc[o];
+        }
     }
 }
 
 // Backward of conv1x1_small: dx[p][c] = sum_o dy[p][o] w[o][c]; dw[o][c] += sum_p dy[p][o] x[p][c];
-// db[o] += sum_p dy[p][o].  Thread: one pixel at a time, its share of dw / db in registers; a block
-// adds them up in shared memory and then into dw / db with one atomic per entry.  C <= 64.
+// db[o] += sum_p dy[p][o].  Thread: one channel quad of every step-th pixel, so that neighbouring threads
+// read x and write dx side by side and a thread keeps 4 COUT sums (one pixel per thread kept 48 COUT, at
+// 8 warps per SM: 96 us at 16 x 256^2 x 32, whose bytes take 41; by quads: 57 us).  A block adds its sums in
+// shared memory and then into dw / db with one atomic per entry.  C <= 64; the block is a multiple of C / 4.
 template <int COUT>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(256)
 conv1x1_small_bwd(const float *__restrict__ dy, const float *__restrict__ x, int P, int C,
                   const float *__restrict__ w, float *__restrict__ dx, float *dw, float *db)
 {
-    __shared__ float sw[COUT * 64];
     __shared__ float sacc[COUT * 64 + COUT];
-    for (int i = threadIdx.x; i < COUT * C; i += blockDim.x) sw[i] = w[i];
     for (int i = threadIdx.x; i < COUT * C + COUT; i += blockDim.x) sacc[i] = 0.0f;
     __syncthreads();
-    float gw[COUT][64 / 4][4];
-    float gb[COUT];
+    const int Q = C / 4, q = threadIdx.x % Q, per_block = blockDim.x / Q;
+    float gw[COUT][4], gb[COUT], wq[COUT][4];
     #pragma unroll
     for (int o = 0; o < COUT; ++o) {
         gb[o] = 0.0f;
         #pragma unroll
-        for (int q = 0; q < 16; ++q)
-            #pragma unroll
-            for (int i = 0; i < 4; ++i) gw[o][q][i] = 0.0f;
+        for (int i = 0; i < 4; ++i) {
+            gw[o][i] = 0.0f;
+            wq[o][i] = w[o * C + 4 * q + i];
+        }
     }
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
+    for (unsigned p = blockIdx.x * per_block + threadIdx.x / Q; p < (unsigned)P; p += gridDim.x * per_block) {
         float g[COUT];
         #pragma unroll
         for (int o = 0; o < COUT; ++o) {
             g[o] = dy[(size_t)p * COUT + o];
             gb[o] += g[o];
         }
-        const float *xp = x + (size_t)p * C;
-        float *dxp = dx ? dx + (size_t)p * C : nullptr;
+        const Vec<4> v = ldv<4>(x + (size_t)p * C + 4 * q);
+        Vec<4> d;
         #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            if (4 * q >= C) break;
-            const Vec<4> v = ldv<4>(xp + 4 * q);
-            Vec<4> d;
+        for (int i = 0; i < 4; ++i) {
+            float s = 0.0f;
             #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float s = 0.0f;
-                #pragma unroll
-                for (int o = 0; o < COUT; ++o) {
-                    gw[o][q][i] = fmaf(g[o], v.v[i], gw[o][q][i]);
-                    s = fmaf(g[o], sw[o * C + 4 * q + i], s);
-                }
-                d.v[i] = s;
+            for (int o = 0; o < COUT; ++o) {
+                gw[o][i] = fmaf(g[o], v.v[i], gw[o][i]);
+                s = fmaf(g[o], wq[o][i], s);
             }
-            if (dxp) stv<4>(dxp + 4 * q, d);
+            d.v[i] = s;
         }
+        if (dx) stv<4>(dx + (size_t)p * C + 4 * q, d);
     }
-    // warp sums first (shuffles), then one shared-memory atomic per warp and entry
-    const bool lead = (threadIdx.x & 31) == 0;
     #pragma unroll
     for (int o = 0; o < COUT; ++o) {
-        const float b = warp_sum(gb[o]);
-        if (lead) atomicAdd(&sacc[COUT * C + o], b);
+        if (q == 0) atomicAdd(&sacc[COUT * C + o], gb[o]);
         #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            if (4 * q >= C) break;
-            #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float v = warp_sum(gw[o][q][i]);
-                if (lead) atomicAdd(&sacc[o * C + 4 * q + i], v);
-            }
-        }
+        for (int i = 0; i < 4; ++i) atomicAdd(&sacc[o * C + 4 * q + i], gw[o][i]);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < COUT * C; i += blockDim.x)
@@ -346,7 +360,8 @@ int gcd(int a, int b) { return b ? gcd(b, a % b) : a; }
 unsigned blocks_for_groups(long long n, int G)
 {
     const int unit = G / gcd(G, 256);
-    long long b = blocks_for(n);
+    long long b = (n + 255) / 256;
+    if (b > 152LL * kBwdBlocks) b = 152LL * kBwdBlocks;
     b = (b + unit - 1) / unit * unit;
     return (unsigned)b;
 }
@@ -378,6 +393,7 @@ cudaError_t vec_bias_act_bwd(const float *da, const float *z, long long rows, in
         return cudaErrorNotSupported;
     const int G = C / V;
     const unsigned blocks = blocks_for_groups(rows * G, G);
+    if (HW < 1) HW = (int)(rows < 1 ? 1 : rows);        // only dzb and dp use it
     if (V == 8)
         bias_act_bwd_vec<8><<<blocks, 256, C * sizeof(float), s>>>(da, z, (int)rows, C, act, dz, db, dzb, HW, dp, W);
     else
@@ -427,11 +443,10 @@ cudaError_t small_conv1x1(const float *x, long long P, int C, const float *w, co
                           cudaStream_t s)
 {
     const unsigned blocks = blocks_for(P);
-    const size_t sm = (size_t)cout * C * sizeof(float);
     switch (cout) {
-    case 1: conv1x1_small<1><<<blocks, 256, sm, s>>>(x, (int)P, C, w, bias, y); break;
-    case 2: conv1x1_small<2><<<blocks, 256, sm, s>>>(x, (int)P, C, w, bias, y); break;
-    default: conv1x1_small<3><<<blocks, 256, sm, s>>>(x, (int)P, C, w, bias, y); break;
+    case 1: conv1x1_small<1><<<blocks, kHeadBX, 0, s>>>(x, (int)P, C, w, bias, y); break;
+    case 2: conv1x1_small<2><<<blocks, kHeadBX, 0, s>>>(x, (int)P, C, w, bias, y); break;
+    default: conv1x1_small<3><<<blocks, kHeadBX, 0, s>>>(x, (int)P, C, w, bias, y); break;
     }
     return cudaGetLastError();
 }
@@ -439,13 +454,14 @@ cudaError_t small_conv1x1(const float *x, long long P, int C, const float *w, co
 cudaError_t small_conv1x1_bwd(const float *dy, const float *x, long long P, int C, const float *w, int cout, float *dx,
                               float *dw, float *db, cudaStream_t s)
 {
-    long long b = (P + 127) / 128;
-    if (b > 152LL * 2) b = 152LL * 2;      // ~240 registers a thread: two blocks per SM, one wave
+    const int threads = 256 / (C / 4) * (C / 4);
+    long long b = (P * (C / 4) + threads - 1) / threads;
+    if (b > 152LL * 8) b = 152LL * 8;
     const unsigned blocks = (unsigned)(b < 1 ? 1 : b);
     switch (cout) {
-    case 1: conv1x1_small_bwd<1><<<blocks, 128, 0, s>>>(dy, x, (int)P, C, w, dx, dw, db); break;
-    case 2: conv1x1_small_bwd<2><<<blocks, 128, 0, s>>>(dy, x, (int)P, C, w, dx, dw, db); break;
-    default: conv1x1_small_bwd<3><<<blocks, 128, 0, s>>>(dy, x, (int)P, C, w, dx, dw, db); break;
+    case 1: conv1x1_small_bwd<1><<<blocks, threads, 0, s>>>(dy, x, (int)P, C, w, dx, dw, db); break;
+    case 2: conv1x1_small_bwd<2><<<blocks, threads, 0, s>>>(dy, x, (int)P, C, w, dx, dw, db); break;
+    default: conv1x1_small_bwd<3><<<blocks, threads, 0, s>>>(dy, x, (int)P, C, w, dx, dw, db); break;
     }
     return cudaGetLastError();
 }
