@@ -74,7 +74,13 @@ struct Epi {
     int act, on;
     const float *zin;
     float *db;
+    bool wide;           // z, a and zin are 32-byte aligned
 };
+
+inline bool aligned32(const void *a, const void *b, const void *c)
+{
+    return ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b) | reinterpret_cast<uintptr_t>(c)) & 31) == 0;
+}
 
 // Warp reduce-scatter of 32 values per lane: afterwards v[0] of lane l is the sum over the warp's lanes
 // of their v[l].  Each of the five steps keeps half of a lane's values and adds its partner's matching
@@ -94,7 +100,15 @@ __device__ __forceinline__ float warp_reduce_scatter32(float v[32], int lane)
     return v[0];
 }
 
-__device__ __forceinline__ float sigm(float v) { return 1.0f / (1.0f + expf(-v)); }
+// 1 / (1 + e^-v), the quotient rounded correctly: see nn_vec.cu.
+__device__ __forceinline__ float sigm(float v)
+{
+    const float d = 1.0f + expf(-v);
+    if (!(d < 4.0e37f)) return 1.0f / d;
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return fmaf(r, fmaf(-d, r, 1.0f), r);
+}
 
 // MT output tiles stacked along y share one halo window per 8-channel plane: (16 MT + 2) rows x 10
 // pixels x 16 B, and every stage's weights.
@@ -251,6 +265,32 @@ __device__ __forceinline__ void teardown(uint32_t tmem)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(COLS));
 }
 
+// Eight floats by one 32-byte access (a whole sector; two of 16 bytes reach the L2 as two half-filled ones) where
+// the address allows it, else by two.
+__device__ __forceinline__ void store8(float *p, const float v[8], bool wide)
+{
+    if (wide) {
+        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]),
+                     "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
+    } else {
+        float4 *q = reinterpret_cast<float4 *>(p);
+        q[0] = make_float4(v[0], v[1], v[2], v[3]);
+        q[1] = make_float4(v[4], v[5], v[6], v[7]);
+    }
+}
+__device__ __forceinline__ void load8(const float *p, float v[8], bool wide)
+{
+    if (wide) {
+        asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                     : "l"(p));
+    } else {
+        const float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    }
+}
+
 // Epilogue of accumulator columns c .. c + 31 of output-channel block n0 for one pixel (yy, xx) of
 // image img (one TMEM lane): plain y = alpha acc + beta y (on == 0), bias + SiLU (on == 1) or the
 // SiLU backward with the bias-gradient sums into sdb (on == 2; every lane of the warp takes part).
@@ -269,20 +309,15 @@ __device__ __forceinline__ void epi_store32(const uint32_t r[32], int c, int n0,
             for (int e = 0; e < 8; ++e) v[j + e] = ok ? __uint_as_float(r[j + e]) : 0.0f;
             if (!ok) continue;
             if (epi.act) {
-                const float4 *zq = reinterpret_cast<const float4 *>(epi.zin + pix * cout + col0 + j);
-                const float4 z0 = zq[0], z1 = zq[1];
-                const float zz[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
+                float zz[8];
+                load8(epi.zin + pix * cout + col0 + j, zz, epi.wide);
                 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     const float sg = sigm(zz[e]);
                     v[j + e] *= sg * (1.0f + zz[e] * (1.0f - sg));
                 }
             }
-            if (epi.z) {
-                float4 *q = reinterpret_cast<float4 *>(epi.z + pix * cout + col0 + j);
-                q[0] = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-                q[1] = make_float4(v[j + 4], v[j + 5], v[j + 6], v[j + 7]);
-            }
+            if (epi.z) store8(epi.z + pix * cout + col0 + j, v + j, epi.wide);
             __half2 h[4];
             #pragma unroll
             for (int e = 0; e < 4; ++e) h[e] = __floats2half2_rn(v[j + 2 * e], v[j + 2 * e + 1]);
@@ -304,20 +339,12 @@ __device__ __forceinline__ void epi_store32(const uint32_t r[32], int c, int n0,
             float v[8];
             #pragma unroll
             for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(r[j + e]) + epi.bias[col0 + j + e];
-            if (epi.z) {
-                float4 *q = reinterpret_cast<float4 *>(epi.z + pix * cout + col0 + j);
-                q[0] = make_float4(v[0], v[1], v[2], v[3]);
-                q[1] = make_float4(v[4], v[5], v[6], v[7]);
-            }
+            if (epi.z) store8(epi.z + pix * cout + col0 + j, v, epi.wide);
             if (epi.act) {
                 #pragma unroll
                 for (int e = 0; e < 8; ++e) v[e] = v[e] * sigm(v[e]);
             }
-            if (epi.a) {
-                float4 *q = reinterpret_cast<float4 *>(epi.a + pix * cout + col0 + j);
-                q[0] = make_float4(v[0], v[1], v[2], v[3]);
-                q[1] = make_float4(v[4], v[5], v[6], v[7]);
-            }
+            if (epi.a) store8(epi.a + pix * cout + col0 + j, v, epi.wide);
             if (epi.ab) {
                 __half2 h[4];
                 #pragma unroll
@@ -329,7 +356,15 @@ __device__ __forceinline__ void epi_store32(const uint32_t r[32], int c, int n0,
         }
         return;
     }
-    if (vec_y && col0 + 32 <= cout) {
+    if (vec_y == 2 && beta == 0.0f && col0 + 32 <= cout) {
+        #pragma unroll
+        for (int j = 0; j < 32; j += 8) {
+            float v[8];
+            #pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = alpha * __uint_as_float(r[j + e]);
+            store8(yrow + col0 + j, v, true);
+        }
+    } else if (vec_y && col0 + 32 <= cout) {
         #pragma unroll
         for (int j = 0; j < 32; j += 4) {
             float4 v = make_float4(alpha * __uint_as_float(r[j]), alpha * __uint_as_float(r[j + 1]),
@@ -858,7 +893,10 @@ cudaError_t launch_conv3_tma_mt(const void *xb, const __half *wp, int N, int H, 
     const int reserve = reserve_stages(nstages, fwd_stage_bytes<TN, MT>(), TN * MT);
     const size_t smem = (size_t)reserve * fwd_stage_bytes<TN, MT>() + 1024;
     dim3 grid((W + kTilePx - 1) / kTilePx, (H + kTileRows * MT - 1) / (kTileRows * MT), N * ntn);
-    const int vec_y = (ldy % 4 == 0) && ((reinterpret_cast<uintptr_t>(y) & 15) == 0);
+    // 16-byte stores, or 32-byte ones (2)
+    const int vec_y = (ldy % 8 == 0) && ((reinterpret_cast<uintptr_t>(y) & 31) == 0)   ? 2
+                      : (ldy % 4 == 0) && ((reinterpret_cast<uintptr_t>(y) & 15) == 0) ? 1
+                                                                                       : 0;
     static bool attr_set = false;       // per instantiation
     if (!attr_set) {
         const int most = (kFwdStages > reserve ? kFwdStages : reserve) * fwd_stage_bytes<TN, MT>() + 1024;
@@ -1087,7 +1125,7 @@ extern "C" int smrt_nn_conv3_tma_bias_act(const void *xb, int N, int H, int W, i
     cudaStream_t s = (cudaStream_t)stream;
     CUresult r = CUDA_SUCCESS;
     const __half *w = (const __half *)wp;
-    const Epi epi{bias, z, a, (__half *)ab, act, 1, nullptr, nullptr};
+    const Epi epi{bias, z, a, (__half *)ab, act, 1, nullptr, nullptr, aligned32(z, a, nullptr)};
     cudaError_t e;
     const int TN = tile_n(cout);
     if (TN == 32) e = launch_conv3_tma<32>(xb, w, N, H, W, C, cout, 1.0f, 0.0f, nullptr, cout, err, s, epi, &r);
@@ -1113,7 +1151,7 @@ extern "C" int smrt_nn_conv3_tma_act_bwd(const void *dzb, int N, int H, int W, i
     cudaStream_t s = (cudaStream_t)stream;
     CUresult r = CUDA_SUCCESS;
     const __half *w = (const __half *)wp;
-    const Epi epi{nullptr, dz, nullptr, (__half *)dzb_out, act, 2, z, db};
+    const Epi epi{nullptr, dz, nullptr, (__half *)dzb_out, act, 2, z, db, aligned32(dz, z, nullptr)};
     cudaError_t e;
     const int TN = tile_n(cout);
     if (TN == 32) e = launch_conv3_tma<32>(dzb, w, N, H, W, C, cout, 1.0f, 0.0f, nullptr, cout, err, s, epi, &r);
