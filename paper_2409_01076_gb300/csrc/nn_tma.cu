@@ -887,12 +887,22 @@ cudaError_t launch_conv3_tma_mt(const void *xb, const __half *wp, int N, int H, 
     if (*map_err != CUDA_SUCCESS) return cudaErrorInvalidValue;
     const int ntn = (cout + TN - 1) / TN;
     const int nchunks = C / kChunk;
-    // a 32-wide single tile with at most two chunks: one stage (15 KB), so that 14 CTAs share an SM and
-    // hide each other's copy latency; otherwise up to four stages per CTA
-    const int nstages = (TN == 32 && MT == 1 && nchunks <= 2) ? 1 : (nchunks < kFwdStages ? nchunks : kFwdStages);
+    dim3 grid((W + kTilePx - 1) / kTilePx, (H + kTileRows * MT - 1) / (kTileRows * MT), N * ntn);
+    // Pipeline stages.  A CTA's copies, MMAs and epilogue follow one another, so what overlaps them is other CTAs
+    // on the SM, and shared memory decides how many: few stages win as soon as the grid can fill the SM with more
+    // CTAs.  Layers at batch 16, us with 4 stages -> as chosen (1 or 2; 3 lies between): 96 -> 32 channels at 256^2
+    // 160 -> 112 (2), 64 -> 64 at 128^2 76 -> 42 (1), 192 -> 64 108 -> 68 (1), 128 -> 128 at 64^2 64 -> 41 (2),
+    // 384 -> 128 91 -> 60 (2).  Two 32-wide chunks fit one stage each; 64-wide tiles take one stage when more CTAs
+    // are waiting than fit with two (128 -> 64 at 64^2: 512 CTAs, 16.8 with two, 17.8 with one); a grid of less
+    // than one 128-wide CTA per SM has nothing to overlap and keeps the deep pipeline.
+    const long long ctas = (long long)grid.x * grid.y * grid.z;
+    int nstages = kFwdStages;
+    if (TN == 32) nstages = nchunks <= 2 ? 1 : 2;
+    else if (TN == 64) nstages = ctas > 4LL * sm_count() ? 1 : 2;
+    else if (MT == 2) nstages = 2;
+    if (nstages > nchunks) nstages = nchunks;
     const int reserve = reserve_stages(nstages, fwd_stage_bytes<TN, MT>(), TN * MT);
     const size_t smem = (size_t)reserve * fwd_stage_bytes<TN, MT>() + 1024;
-    dim3 grid((W + kTilePx - 1) / kTilePx, (H + kTileRows * MT - 1) / (kTileRows * MT), N * ntn);
     // 16-byte stores, or 32-byte ones (2)
     const int vec_y = (ldy % 8 == 0) && ((reinterpret_cast<uintptr_t>(y) & 31) == 0)   ? 2
                       : (ldy % 4 == 0) && ((reinterpret_cast<uintptr_t>(y) & 15) == 0) ? 1
