@@ -54,7 +54,7 @@ constexpr int kPlane = kHaloRows * kHaloPx * 16;           // 2,880 B: one halo 
 constexpr int kDzPlane = kTileRows * kTilePx * 16;         // 2,048 B: one 8-channel plane of dz
 constexpr int kFwdStages = 4;
 constexpr int kWgStages = 6;
-constexpr int kWgTN = 32;                                  // output channels per weight-gradient CTA
+constexpr int kWgTN = 32;                                  // output channels per weight-gradient CTA (or 64)
 constexpr int kWgPlanes = 16;                              // input channels per weight-gradient CTA / 8
 constexpr unsigned long long kWaitNs = 1000000000ull;      // a wait gives up after 1 s (%globaltimer)
 
@@ -478,27 +478,37 @@ conv3_tma_kernel(const __grid_constant__ CUtensorMap tmx, const __half *__restri
 }
 
 // ---- weight gradient -------------------------------------------------------------------------
-// grid (input-channel blocks of 128 x output-channel blocks of 32, pixel-tile splits).  A CTA
-// accumulates D_t[c][o] = sum over its pixel tiles of x(p + tap t)[c] dz(p)[o] for all nine taps
-// (9 x 32 TMEM columns), then adds alpha D_t into gw[o][t*C + c] with float32 atomics.
+// grid (input-channel blocks of 128 x output-channel blocks of TN, pixel-tile splits).  A CTA
+// accumulates D_t[c][o] = sum over its pixel tiles of x(p + tap t)[c] dz(p)[o] for its taps t (TN TMEM columns
+// each), then adds alpha D_t into gw[o][t*C + c] with float32 atomics.
+// TN = 32: all nine taps (288 columns).  An MMA of 128 x 32 x 16 reads 5 KB of shared memory for 16 clocks of
+// tensor work, and issues no faster than one of 128 x 64 x 16, so where cout is a multiple of 64, TN = 64: half
+// the MMAs, in two kinds of CTA that take taps 0-4 and 5-8 (320 and 256 of the 512 columns) and split the pixel
+// tiles 5 : 4.
+template <int TN>
 __global__ void __launch_bounds__(128)
 conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmz, int H, int W,
-                   int C, int cout, int tiles_x, int tiles_y, int ntiles, int nbk, int per, int planes, int nstages,
-                   int stage_bytes, float alpha, float *gw, int ldg, int *err)
+                   int C, int cout, int tiles_x, int tiles_y, int ntiles, int nbk, int split0, int per0, int per1,
+                   int planes, int nstages, int stage_bytes, float alpha, float *gw, int ldg, int *err)
 {
     extern __shared__ unsigned char dyn_raw[];
     __shared__ __align__(8) unsigned long long full[kWgStages], empty[kWgStages], done;
     __shared__ uint32_t tmem_holder;
     __shared__ int failed;
-    constexpr uint32_t kCols = 512;         // 9 taps x 32 columns, rounded up to a power of two
+    constexpr uint32_t kCols = 512;         // 9 x 32 or 5 x 64 columns, rounded up to a power of two
+    constexpr int kZ = TN / 8;              // dz planes of a tile
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int mb = blockIdx.x / nbk, nb = blockIdx.x % nbk;
-    const int t_beg = blockIdx.y * per;
+    // CTAs [0, split0) of a channel block take the first taps, the others the rest
+    const bool second = (int)blockIdx.y >= split0;
+    const int tap0 = second ? 5 : 0, tap1 = (TN == 64 && !second) ? 5 : 9;
+    const int per = second ? per1 : per0;
+    const int t_beg = ((int)blockIdx.y - (second ? split0 : 0)) * per;
     const int t_end = min(ntiles, t_beg + per);
     if (t_beg >= t_end) return;             // uniform over the CTA
     const int a_bytes = (planes * kPlane + 127) / 128 * 128;
-    const uint32_t tx = (uint32_t)(planes * kPlane + 4 * kDzPlane);
+    const uint32_t tx = (uint32_t)(planes * kPlane + kZ * kDzPlane);
     const uint32_t base = (smem_u32(dyn_raw) + 1023u) & ~1023u;
 
     const uint32_t tmem = setup<kCols>(&tmem_holder, full, empty, &done, nstages, &failed);
@@ -517,7 +527,7 @@ conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constan
             const uint32_t st = base + (uint32_t)(s * stage_bytes), fb = smem_u32(&full[s]);
             expect_tx(fb, tx);
             tma_load_4d(st, &tmx, 8 * (x0 - 1), y0 - 1, kWgPlanes * mb, img, fb);
-            tma_load_4d(st + a_bytes, &tmz, 8 * x0, y0, 4 * nb, img, fb);
+            tma_load_4d(st + a_bytes, &tmz, 8 * x0, y0, kZ * nb, img, fb);
         }
     } else if (warp == 1 && lane == 0) {
         for (int it = 0; it < n_it; ++it) {
@@ -526,14 +536,14 @@ conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constan
             asm volatile("tcgen05.fence::after_thread_sync;");
             const uint32_t st = base + (uint32_t)(s * stage_bytes);
             #pragma unroll 1
-            for (int t = 0; t < 9; ++t) {
+            for (int t = tap0; t < tap1; ++t) {
                 const int ky = t / 3, kx = t % 3;
                 #pragma unroll
                 for (int j = 0; j < kTileRows / 2; ++j) {        // K = 16 pixels: image rows 2j, 2j + 1
-                    mma_f16(tmem + (uint32_t)(t * kWgTN),
+                    mma_f16(tmem + (uint32_t)((t - tap0) * TN),
                             desc(st + (uint32_t)(((2 * j + ky) * kHaloPx + kx) * 16), kHaloPx * 16, kPlane),
                             desc(st + (uint32_t)a_bytes + (uint32_t)(2 * j * 128), 128, kDzPlane),
-                            idesc<kWgTN, true>(), (it > 0 || j > 0) ? 1u : 0u);
+                            idesc<TN, true>(), (it > 0 || j > 0) ? 1u : 0u);
                 }
             }
             commit(smem_u32(&empty[s]));
@@ -548,15 +558,18 @@ conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constan
     if (!failed) {
         const int c = kWgPlanes * 8 * mb + warp * 32 + lane;
         #pragma unroll 1
-        for (int t = 0; t < 9; ++t) {
-            uint32_t r[32];
-            tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(t * kWgTN), r);
-            if (c >= C) continue;
-            float *g = gw + (size_t)t * C + c;
-            #pragma unroll
-            for (int j = 0; j < kWgTN; ++j) {
-                const int o = kWgTN * nb + j;
-                if (o < cout) atomicAdd(g + (size_t)o * ldg, alpha * __uint_as_float(r[j]));
+        for (int t = tap0; t < tap1; ++t) {
+            #pragma unroll 1
+            for (int o0 = 0; o0 < TN; o0 += 32) {
+                uint32_t r[32];
+                tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((t - tap0) * TN + o0), r);
+                if (c >= C) continue;
+                float *g = gw + (size_t)t * C + c;
+                #pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const int o = TN * nb + o0 + j;
+                    if (o < cout) atomicAdd(g + (size_t)o * ldg, alpha * __uint_as_float(r[j]));
+                }
             }
         }
     }
@@ -1243,18 +1256,21 @@ extern "C" int smrt_nn_conv3_wgrad_tma(const void *xb, int N, int H, int W, int 
         return tma_fail(SMRT_ERR_CUDA, "smrt_nn_conv3_wgrad_tma: tensor map rejected (%d)", (int)r);
 
     if (C == 16 || C == 32) return wgrad_grouped(xb, N, H, W, C, dzb, cout, alpha, gw, ldg, err, stream, tmz);
-    const int mbk = (C + 8 * kWgPlanes - 1) / (8 * kWgPlanes), nbk = (cout + kWgTN - 1) / kWgTN;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148;
+    const int TN = cout % 64 == 0 ? 64 : kWgTN;
+    if (TN == 64) r = blocked_map(&tmz, dzb, N, H, W, cout, kTilePx, kTileRows, 8);
+    if (r != CUDA_SUCCESS)
+        return tma_fail(SMRT_ERR_CUDA, "smrt_nn_conv3_wgrad_tma: tensor map rejected (%d)", (int)r);
+    const int mbk = (C + 8 * kWgPlanes - 1) / (8 * kWgPlanes), nbk = (cout + TN - 1) / TN;
     // one CTA per SM (each holds all 512 TMEM columns): split the pixel tiles to fill the SMs
-    long long splits = sms / (mbk * nbk);
-    if (splits < 1) splits = 1;
-    if (splits > ntiles) splits = ntiles;
-    const int per = (int)((ntiles + splits - 1) / splits);
-    splits = (ntiles + per - 1) / per;
+    const int kinds = TN == 64 ? 2 : 1;
+    long long splits = sm_count() / (mbk * nbk);
+    if (splits < kinds) splits = kinds;
+    long long split0 = TN == 64 ? (5 * splits + 4) / 9 : splits, split1 = splits - split0;
+    if (split0 > ntiles) split0 = ntiles;
+    if (split1 > ntiles) split1 = ntiles;
+    const int per0 = (int)((ntiles + split0 - 1) / split0), per1 = split1 ? (int)((ntiles + split1 - 1) / split1) : 1;
     const int a_bytes = (planes * kPlane + 127) / 128 * 128;
-    const int stage = (a_bytes + 4 * kDzPlane + 1023) / 1024 * 1024;
+    const int stage = (a_bytes + TN / 8 * kDzPlane + 1023) / 1024 * 1024;
     const int a_reach = kWgPlanes * kPlane;         // the MMA's 128 rows read 16 planes from a stage start
     int nstages = kWgStages;
     auto need = [&](int n) { return (size_t)(n - 1) * stage + (size_t)(stage > a_reach ? stage : a_reach + 128); };
@@ -1263,17 +1279,17 @@ extern "C" int smrt_nn_conv3_wgrad_tma(const void *xb, int N, int H, int W, int 
     if (smem < 120 * 1024) smem = 120 * 1024;       // keeps a second CTA (and its TMEM request) off the SM
     if (smem > 220 * 1024 || mbk * nbk > 65535 || splits > 65535)
         return tma_fail(SMRT_ERR_ARG, "smrt_nn_conv3_wgrad_tma: sizes out of range (C %d cout %d)", C, cout);
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(conv3_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             220 * 1024);
+    auto kernel = TN == 64 ? conv3_wgrad_kernel<64> : conv3_wgrad_kernel<32>;
+    static bool attr_set[2] = {false, false};
+    if (!attr_set[kinds - 1]) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         if (e != cudaSuccess) return tma_fail(SMRT_ERR_CUDA, "smrt_nn_conv3_wgrad_tma: %s", cudaGetErrorString(e));
-        attr_set = true;
+        attr_set[kinds - 1] = true;
     }
-    dim3 grid(mbk * nbk, (unsigned)splits);
-    conv3_wgrad_kernel<<<grid, 128, smem, (cudaStream_t)stream>>>(tmx, tmz, H, W, C, cout, tiles_x, tiles_y,
-                                                                  (int)ntiles, nbk, per, planes, nstages, stage, alpha,
-                                                                  gw, ldg, err);
+    dim3 grid(mbk * nbk, (unsigned)(split0 + split1));
+    kernel<<<grid, 128, smem, (cudaStream_t)stream>>>(tmx, tmz, H, W, C, cout, tiles_x, tiles_y, (int)ntiles, nbk,
+                                                      (int)split0, per0, per1, planes, nstages, stage, alpha, gw, ldg,
+                                                      err);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return tma_fail(SMRT_ERR_CUDA, "smrt_nn_conv3_wgrad_tma: %s", cudaGetErrorString(e));
     return SMRT_OK;
