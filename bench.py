@@ -196,18 +196,18 @@ def measured_hbm_peak():
 
 
 def kernel_source_hash():
-    """Hash of the sources the step kernel is compiled from."""
+    """Hash of the sources the update kernels are compiled from."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2409_01076_gb300", "csrc")
     for name in sorted(os.listdir(csrc)):
-        if name in ("d2q9.cuh", "kernels.cuh") or (name.startswith("prec_") and name.endswith(".cu")):
+        if name in ("d2q9.cuh", "kernels.cuh", "sweep.cuh") or (name.startswith("prec_") and name.endswith(".cu")):
             with open(os.path.join(csrc, name), "rb") as fh:
                 h.update(name.encode() + b"\0" + fh.read())
     return h.hexdigest()[:16]
 
 
 def committed_traffic(prec, layout, kind):
-    """DRAM bytes per node update of the step kernel from the committed ncu summary, if it
+    """DRAM bytes per node and launch of the update kernel from the committed ncu summary, if it
     was taken on the current kernel sources (else None)."""
     path = os.path.join(ROOT, "profiles", "step_kernel_traffic.md")
     try:
@@ -228,6 +228,17 @@ def committed_traffic(prec, layout, kind):
 
 
 # ---- the GPU arm ---------------------------------------------------------------------
+
+def update_launches(steps, nodes, prec, layout):
+    """Update kernels that smrt_step(steps) launches.  The two-buffer layout of a float format takes up to
+    three updates per pass over the state (the last ones by twos); a lattice of at most 600^2 nodes up to
+    eight, in tiles (then a lower bound); every other update is a launch of its own."""
+    if layout != "ab" or steps < 2:
+        return steps
+    if nodes <= 600 * 600:
+        return -(-steps // 8)
+    return steps if prec == "f64" else -(-steps // 3)
+
 
 def make_handle(S, wl, prec, layout, kind, check=True):
     """prec: f64, f32, f16 or bf16, with "-sr" for stochastic rounding of the 16-bit formats."""
@@ -265,9 +276,10 @@ def run_variant(S, wl, rho_d, u_d, prec, layout, kind, steps, warmup, world):
     S.smrt_destroy(h)
     nodes = wl["nx"] * wl["ny"]
     mlups = nodes * steps / (ms * 1e-3) / 1e6
+    launches = update_launches(steps, nodes, prec, layout)
     return {"mlups": round(mlups, 1), "ms_per_step": round(ms / steps, 5),
-            "hbm_gbs": round(BYTES_PER_NODE[prec.replace("-sr", "")] * nodes / (ms / steps * 1e-3) / 1e9, 1),
-            "steps": steps}
+            "hbm_gbs": round(BYTES_PER_NODE[prec.replace("-sr", "")] * nodes * launches / (ms * 1e-3) / 1e9, 1),
+            "steps": steps, "launches": launches}
 
 
 def host_link_gbs(host, reps=3):
@@ -518,7 +530,8 @@ def gpu_arm(args):
     ms = max_over_ranks(ms, world)
     sec = ms * 1e-3
     mlups = world * nodes * args.steps / sec / 1e6
-    per_launch = sec / args.steps
+    launches = update_launches(args.steps, nodes, args.prec, args.layout)
+    per_launch = sec / launches
     peak, peak_src = measured_hbm_peak()
     achieved = BYTES_PER_NODE[args.prec.replace("-sr", "")] * nodes / per_launch / 1e9
     traffic_per_node, _ = committed_traffic(args.prec, args.layout, args.kind)
@@ -538,8 +551,10 @@ def gpu_arm(args):
                      if peak_src == "measured" else "fallback 6.8 TB/s",
                      "traffic": (round(traffic_per_node * nodes) if traffic_per_node else None),
                      "algorithmic_bytes_per_launch": BYTES_PER_NODE[args.prec.replace("-sr", "")] * nodes,
-                     "kernel": "step_kernel<%s,%s,%s>" % (args.prec, args.kind, args.layout)},
-        "gpu_launches": args.steps,
+                     "updates_per_launch": round(args.steps / launches, 3),
+                     "kernel": "%s<%s,%s,%s>" % ("step_kernel" if launches == args.steps else "sweep_kernel", args.prec,
+                                                 args.kind, args.layout)},
+        "gpu_launches": launches,
         "clocks": clk,
         "check": {"residual_after": r, "mass_rel_err": abs(sums[0] / nodes - 1.0)},
     }

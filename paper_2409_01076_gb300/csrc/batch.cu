@@ -131,6 +131,7 @@ batch_sweep_kernel(const float *src, float *dst, const BatchSweep *__restrict__ 
     using Shared = SweepShared<float, T>;
     Shared &sm = *reinterpret_cast<Shared *>(sweep_smem);
     Raw4<float> *seam = reinterpret_cast<Raw4<float> *>(sweep_smem + sizeof(Shared));
+    follow_predecessor();
     if ((int)blockIdx.x >= counts[3]) return;
     const int2 w = items[blockIdx.x];
     const unsigned long long *g = reinterpret_cast<const unsigned long long *>(sw + w.x);
@@ -156,8 +157,7 @@ cudaError_t launch_batch_sweep_kt(const float *src, float *dst, const void *sw, 
     const CollideConsts cc = collide_consts<KIND>(make_params<float>(hp));
     const size_t smem = sizeof(SweepShared<float, T>) + (seam ? 9 * 32 * sizeof(Raw4<float>) : 0);
     auto kernel = seam ? batch_sweep_kernel<KIND, T, true> : batch_sweep_kernel<KIND, T, false>;
-    kernel<<<n, 32, smem, s>>>(src, dst, (const BatchSweep *)sw, items, counts, cc);
-    return cudaGetLastError();
+    return launch_following(kernel, (unsigned)n, 32, smem, s, src, dst, (const BatchSweep *)sw, items, counts, cc);
 }
 
 cudaError_t launch_batch_sweep(int kind, int updates, const void *src, void *dst, const void *sw, const int2 *items,

@@ -378,6 +378,7 @@ __global__ void __launch_bounds__(BX)
 step_kernel(const typename Prec<PREC>::R *src, typename Prec<PREC>::R *dst,
             const Params<typename Prec<PREC>::C> p, const StepGeom geo)
 {
+    follow_predecessor();
     step_block<PREC, KIND, MODE, VEC, BX, true, false, SR>(src, dst, p, geo, blockIdx.x);
 }
 
@@ -913,15 +914,12 @@ cudaError_t launch_step_km(const void *src, void *dst, const HostParams &hp, cud
     if (blocks <= 0) return cudaSuccess;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     if constexpr (PREC == SMRT_PREC_F16 || PREC == SMRT_PREC_BF16) {
-        if (hp.rounding == SMRT_ROUND_STOCHASTIC) {
-            step_kernel<PREC, KIND, MODE, VEC, BX, true><<<(unsigned)blocks, BX, 0, s>>>(
-                (const R *)src, (R *)dst, p, geo);
-            return cudaGetLastError();
-        }
+        if (hp.rounding == SMRT_ROUND_STOCHASTIC)
+            return launch_following(step_kernel<PREC, KIND, MODE, VEC, BX, true>, (unsigned)blocks, BX, 0, s,
+                                    (const R *)src, (R *)dst, p, geo);
     }
-    step_kernel<PREC, KIND, MODE, VEC, BX><<<(unsigned)blocks, BX, 0, s>>>(
-        (const R *)src, (R *)dst, p, geo);
-    return cudaGetLastError();
+    return launch_following(step_kernel<PREC, KIND, MODE, VEC, BX>, (unsigned)blocks, BX, 0, s, (const R *)src, (R *)dst,
+                            p, geo);
 }
 
 template <int PREC, int KIND>
@@ -965,8 +963,7 @@ cudaError_t launch_sweep_kt(const void *src, void *dst, const HostParams &hp, cu
         if (hp.rounding == SMRT_ROUND_STOCHASTIC)
             kernel = seam ? sweep_kernel<PREC, KIND, true, T, true> : sweep_kernel<PREC, KIND, true, T, false>;
     }
-    kernel<<<nb, 32, smem, s>>>((const R *)src, (R *)dst, p, cc, salt, strips, rows);
-    return cudaGetLastError();
+    return launch_following(kernel, nb, 32, smem, s, (const R *)src, (R *)dst, p, cc, salt, strips, rows);
 }
 
 template <int PREC, int KIND>
@@ -1000,16 +997,12 @@ cudaError_t launch_tile_k(const TilePlan &t, const void *src, void *dst, const H
     TileSalts salt;
     for (int m = 0; m < kTileMaxT; ++m) salt.s[m] = sr_salt(hp.t + m);
     const unsigned nb = (unsigned)(t.tiles_x * t.tiles_y);
+    auto kernel = tile_kernel<PREC, KIND, false>;
     if constexpr (PREC == SMRT_PREC_F16 || PREC == SMRT_PREC_BF16) {
-        if (hp.rounding == SMRT_ROUND_STOCHASTIC) {
-            tile_kernel<PREC, KIND, true><<<nb, t.threads, t.shared, s>>>((const R *)src, (R *)dst, p, salt, t.W, t.H, t.T,
-                                                                         t.tiles_x);
-            return cudaGetLastError();
-        }
+        if (hp.rounding == SMRT_ROUND_STOCHASTIC) kernel = tile_kernel<PREC, KIND, true>;
     }
-    tile_kernel<PREC, KIND, false><<<nb, t.threads, t.shared, s>>>((const R *)src, (R *)dst, p, salt, t.W, t.H, t.T,
-                                                                  t.tiles_x);
-    return cudaGetLastError();
+    return launch_following(kernel, nb, (unsigned)t.threads, t.shared, s, (const R *)src, (R *)dst, p, salt, t.W, t.H,
+                            t.T, t.tiles_x);
 }
 
 template <int PREC>

@@ -415,6 +415,7 @@ sweep_kernel(const typename Prec<PREC>::R *src, typename Prec<PREC>::R *dst,
     Raw4<typename Prec<PREC>::R> *seam = reinterpret_cast<Raw4<typename Prec<PREC>::R> *>(sweep_smem + sizeof(Shared));
     const int seg = blockIdx.x / strips, strip = blockIdx.x - seg * strips;
     const int r0 = seg * rows;
+    follow_predecessor();
     sweep<PREC, KIND, SR, T, SEAM>(src, dst, p, cc, salt, strip, r0, min(r0 + rows, p.ny), sm, seam);
 }
 

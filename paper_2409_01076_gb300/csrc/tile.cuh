@@ -36,6 +36,7 @@ tile_kernel(const typename Prec<PREC>::R *__restrict__ src, typename Prec<PREC>:
     const int ty = blockIdx.x / tiles_x, x0 = (blockIdx.x - ty * tiles_x) * W, y0 = ty * H;
     const bool wall_x = !p.periodic_x, wall_y = !p.periodic_y;
     bool bad = false;
+    follow_predecessor();
     for (int m = 0; m < T; ++m) {
         // nodes of this update: T - 1 - m rings, as far as the lattice has them
         const int ring = T - 1 - m;
