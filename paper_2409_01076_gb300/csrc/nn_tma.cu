@@ -185,6 +185,13 @@ __device__ __forceinline__ void expect_tx(uint32_t mb, uint32_t bytes)
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(mb), "r"(bytes) : "memory");
 }
 
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t mbar)
+{
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
+                 "[%1, {%2, %3}], [%4];"
+                 :: "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(mbar) : "memory");
+}
+
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2, int c3,
                                             uint32_t mbar)
 {
@@ -394,8 +401,9 @@ __device__ __forceinline__ void epi_store32(const uint32_t r[32], int c, int n0,
 // from one 34-row halo window, so each stage's weights serve twice the pixels.
 template <int TN, int MT>
 __global__ void __launch_bounds__(128)
-conv3_tma_kernel(const __grid_constant__ CUtensorMap tmx, const __half *__restrict__ wp, int H, int W, int C,
-                 int cout, int ntn, int nstages, float alpha, float beta, float *y, int ldy, int vec_y, int *err,
+conv3_tma_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmw,
+                 const __half *__restrict__ wp, int H, int W, int C,
+                 int cout, int ntn, int tnp, int nstages, float alpha, float beta, float *y, int ldy, int vec_y, int *err,
                  Epi epi, unsigned long long wait_ns, int withhold)
 {
     extern __shared__ unsigned char dyn_raw[];
@@ -429,7 +437,8 @@ conv3_tma_kernel(const __grid_constant__ CUtensorMap tmx, const __half *__restri
             const uint32_t st = base + (uint32_t)(s * kSB), fb = smem_u32(&full[s]);
             expect_tx(fb, kTx);
             tma_load_4d(st, &tmx, 8 * (x0 - 1), y0 - 1, 2 * i, img, fb);       // planes 2i, 2i + 1
-            bulk_load(st + kA, wblk + (size_t)i * 18 * TN * 8, 18 * TN * 16, fb);
+            if (tnp == TN) bulk_load(st + kA, wblk + (size_t)i * 18 * TN * 8, 18 * TN * 16, fb);
+            else tma_load_2d(st + kA, &tmw, n0 % tnp * 8, (n0 / tnp * nchunks + i) * 18, fb);   // TN of 18 slabs' rows
         }
     } else if (warp == 1 && lane == 0) {
         for (int i = 0; i < nchunks; ++i) {
@@ -860,6 +869,20 @@ CUresult blocked_map(CUtensorMap *map, const void *xb, int N, int H, int W, int 
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
+// Packed weights (tnp-wide tiles) as rows of one slab each: a box is `rows` output channels of 18 slabs.
+CUresult weight_map(CUtensorMap *map, const void *wp, int tnp, long long slabs, int rows)
+{
+    EncodeTiledFn enc = encode_tiled();
+    if (!enc) return CUDA_ERROR_NOT_SUPPORTED;
+    const cuuint64_t dim[2] = {8ull * tnp, (cuuint64_t)slabs};
+    const cuuint64_t str[1] = {16ull * tnp};
+    const cuuint32_t box[2] = {(cuuint32_t)(8 * rows), 18};
+    const cuuint32_t ones[2] = {1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void *>(wp), dim, str, box, ones,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+}
+
 bool blocked_args_ok(const void *p, int N, int H, int W, int C)
 {
     return p && N >= 1 && H >= 1 && W >= 1 && C >= 8 && C % 8 == 0 && (reinterpret_cast<uintptr_t>(p) & 15) == 0 &&
@@ -893,13 +916,18 @@ int reserve_stages(int nstages, int stage_bytes, int tmem_cols)
 template <int TN, int MT>
 cudaError_t launch_conv3_tma_mt(const void *xb, const __half *wp, int N, int H, int W, int C, int cout, float alpha,
                                 float beta, float *y, int ldy, int *err, cudaStream_t s, const Epi &epi,
-                                unsigned long long wait_ns, int withhold, CUresult *map_err)
+                                unsigned long long wait_ns, int withhold, CUresult *map_err, int tnp = TN)
 {
     CUtensorMap tmx;
     *map_err = blocked_map(&tmx, xb, N, H, W, C, kHaloPx, kTileRows * MT + 2, 2);
     if (*map_err != CUDA_SUCCESS) return cudaErrorInvalidValue;
     const int ntn = (cout + TN - 1) / TN;
     const int nchunks = C / kChunk;
+    CUtensorMap tmw = tmx;                  // read only by tiles narrower than the packing
+    if (tnp != TN) {
+        *map_err = weight_map(&tmw, wp, tnp, (long long)((cout + tnp - 1) / tnp) * nchunks * 18, TN);
+        if (*map_err != CUDA_SUCCESS) return cudaErrorInvalidValue;
+    }
     dim3 grid((W + kTilePx - 1) / kTilePx, (H + kTileRows * MT - 1) / (kTileRows * MT), N * ntn);
     // Pipeline stages.  A CTA's copies, MMAs and epilogue follow one another, so what overlaps them is other CTAs
     // on the SM, and shared memory decides how many: few stages win as soon as the grid can fill the SM with more
@@ -910,7 +938,8 @@ cudaError_t launch_conv3_tma_mt(const void *xb, const __half *wp, int N, int H, 
     // than one 128-wide CTA per SM has nothing to overlap and keeps the deep pipeline.
     const long long ctas = (long long)grid.x * grid.y * grid.z;
     int nstages = kFwdStages;
-    if (TN == 32) nstages = nchunks <= 2 ? 1 : 2;
+    if (ctas <= sm_count()) nstages = kFwdStages;
+    else if (TN == 32) nstages = nchunks <= 2 ? 1 : 2;
     else if (TN == 64) nstages = ctas > 4LL * sm_count() ? 1 : 2;
     else if (MT == 2) nstages = 2;
     if (nstages > nchunks) nstages = nchunks;
@@ -928,7 +957,7 @@ cudaError_t launch_conv3_tma_mt(const void *xb, const __half *wp, int N, int H, 
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    conv3_tma_kernel<TN, MT><<<grid, 128, smem, s>>>(tmx, wp, H, W, C, cout, ntn, nstages, alpha, beta, y, ldy,
+    conv3_tma_kernel<TN, MT><<<grid, 128, smem, s>>>(tmx, tmw, wp, H, W, C, cout, ntn, tnp, nstages, alpha, beta, y, ldy,
                                                      vec_y, err, epi, wait_ns, withhold);
     return cudaGetLastError();
 }
@@ -943,6 +972,15 @@ cudaError_t launch_conv3_tma(const void *xb, const __half *wp, int N, int H, int
                              float beta, float *y, int ldy, int *err, cudaStream_t s, const Epi &epi,
                              CUresult *map_err, unsigned long long wait_ns = kWaitNs, int withhold = 0)
 {
+    // A single image leaves most SMs without a tile: 32-wide tiles of the same packed weights, whose box of one TMA
+    // copy they are.  The sums of a pixel and channel are the same.
+    if constexpr (TN > 32) {
+        const long long ctas = (long long)((W + kTilePx - 1) / kTilePx) * ((H + kTileRows - 1) / kTileRows) * N *
+                               ((cout + TN - 1) / TN);
+        if (2 * ctas <= sm_count())
+            return launch_conv3_tma_mt<32, 1>(xb, wp, N, H, W, C, cout, alpha, beta, y, ldy, err, s, epi, wait_ns,
+                                              withhold, map_err, TN);
+    }
     if constexpr (TN == 128) {
         const long long cols = (long long)((W + kTilePx - 1) / kTilePx) * N * ((cout + TN - 1) / TN);
         const long long tiles = cols * ((H + kTileRows - 1) / kTileRows);
