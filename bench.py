@@ -232,12 +232,15 @@ def committed_traffic(prec, layout, kind):
 def update_launches(steps, nodes, prec, layout):
     """Update kernels that smrt_step(steps) launches.  The two-buffer layout of a float format takes up to
     three updates per pass over the state (the last ones by twos); a lattice of at most 600^2 nodes up to
-    eight, in tiles (then a lower bound); every other update is a launch of its own."""
+    eight, in tiles (then a lower bound); every other update is a launch of its own, and so is every one of
+    stochastic rounding but to BF16 from 4096^2 nodes on."""
     if layout != "ab" or steps < 2:
         return steps
     if nodes <= 600 * 600:
         return -(-steps // 8)
-    return steps if prec == "f64" else -(-steps // 3)
+    if prec in ("f64", "f16-sr") or (prec == "bf16-sr" and nodes < 4096 * 4096):
+        return steps
+    return -(-steps // 3)
 
 
 def make_handle(S, wl, prec, layout, kind, check=True):
@@ -634,7 +637,7 @@ def batched_throughput(S, steps, layout="ab", count=512, sides=(64, 128, 256, 51
     after = int((S.smrt_batch_status(b)[2] == S.SMRT_BATCH_ACTIVE).sum())
     S.smrt_batch_destroy(b)
     return {"mlups": round(nodes * steps / (ms * 1e-3) / 1e6, 1), "ms_per_step": round(ms / steps, 5),
-            "hbm_gbs": round(72 * nodes / (ms / steps * 1e-3) / 1e9, 1), "steps": steps, "cavities": len(cav),
+            "steps": steps, "cavities": len(cav),
             "active": int(active.sum()), "active_after": after, "re": list(re),
             "nodes": nodes, "tile_shape_choice": choice, "layout": layout}
 

@@ -97,18 +97,34 @@ template <> struct Prec<SMRT_PREC_F32> {
 // that.  IEEE half keeps 10 of float's 23 mantissa bits where it is normal (|c| >= 2^-14): add 13 of
 // the bits below them and truncate; below that its spacing is fixed at 2^-24, so a uniform fraction
 // of 2^-24 is added before truncating.  Truncation is toward zero on the magnitude, so the rounding
-// is symmetric in the sign.
+// is symmetric in the sign.  The fraction is made in the FP32 pipe: 2^23 + r is an OR, and the product
+// r 2^-40 is exact, so one multiply-add rounds as the separate addition would.  (Converting r as an
+// integer took the quarter-rate conversion unit once per population: without it 8192^2 in place went
+// from 129.8k to 134.6k MLUPS, three updates per pass from 124.7k to 136.0k.)
+// to_r2_sr rounds two values into one packed word (a below b), the same bits as two calls of to_r_sr.
 template <> struct Prec<SMRT_PREC_F16> {
     using R = unsigned short;
     using C = float;
     static constexpr bool kExactWeights = false;
     static __device__ __forceinline__ C to_c(R r) { return __half2float(__ushort_as_half(r)); }
     static __device__ __forceinline__ R to_r(C c) { return __half_as_ushort(__float2half_rn(c)); }
-    static __device__ __forceinline__ R to_r_sr(C c, uint32_t r)
+    // c and its dither: truncating this to half is the stochastic rounding of c
+    static __device__ __forceinline__ float dithered(C c, uint32_t r)
     {
         const float yn = __uint_as_float(__float_as_uint(c) + (r & 0x1FFFu));
-        const float ys = c + copysignf(__uint_as_float(0x33800000u) * ((float)(r & 0xFFFFu) * (1.0f / 65536.0f)), c);
-        return __half_as_ushort(__float2half_rz(fabsf(c) >= 6.103515625e-05f ? yn : ys));
+        const float u = __uint_as_float(0x4B000000u | (r & 0xFFFFu)) - 8388608.0f;
+        const float ys = fmaf(u, copysignf(0x1p-40f, c), c);
+        return fabsf(c) >= 6.103515625e-05f ? yn : ys;
+    }
+    static __device__ __forceinline__ R to_r_sr(C c, uint32_t r)
+    {
+        return __half_as_ushort(__float2half_rz(dithered(c, r)));
+    }
+    static __device__ __forceinline__ uint32_t to_r2_sr(C a, C b, uint32_t ra, uint32_t rb)
+    {
+        uint32_t d;
+        asm("cvt.rz.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(dithered(b, rb)), "f"(dithered(a, ra)));
+        return d;
     }
 };
 template <> struct Prec<SMRT_PREC_BF16> {
@@ -120,6 +136,10 @@ template <> struct Prec<SMRT_PREC_BF16> {
     static __device__ __forceinline__ R to_r_sr(C c, uint32_t r)
     {
         return (R)((__float_as_uint(c) + (r & 0xFFFFu)) >> 16);
+    }
+    static __device__ __forceinline__ uint32_t to_r2_sr(C a, C b, uint32_t ra, uint32_t rb)
+    {
+        return __byte_perm(__float_as_uint(a) + (ra & 0xFFFFu), __float_as_uint(b) + (rb & 0xFFFFu), 0x7632);
     }
 };
 

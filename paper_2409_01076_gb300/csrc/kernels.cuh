@@ -368,7 +368,17 @@ __device__ __forceinline__ void step_block(const typename Prec<PREC>::R *src, ty
         R *rp = dst + (size_t)plane * (size_t)p.plane + (size_t)row * (size_t)p.pitch;
         R vals[VEC];
         #pragma unroll
-        for (int k = 0; k < VEC; ++k) vals[k] = round_store<PREC, SR>(g[k][a], nh[k], a);
+        for (int k = 0; k < VEC; ++k) {
+            if constexpr (SR && VEC % 2 == 0) {
+                if (k % 2) continue;
+                const uint32_t two = Prec<PREC>::to_r2_sr(g[k][a], g[k + 1][a], sr_pop_bits(nh[k], a),
+                                                          sr_pop_bits(nh[k + 1], a));
+                vals[k] = (R)two;
+                vals[k + 1] = (R)(two >> 16);
+            } else {
+                vals[k] = round_store<PREC, SR>(g[k][a], nh[k], a);
+            }
+        }
         store_row<R, VEC>(rp, i0, s, lane, active, vals, seg);
     }
 }
@@ -959,7 +969,10 @@ cudaError_t launch_sweep_kt(const void *src, void *dst, const HostParams &hp, cu
     const bool seam = p.periodic_x && hp.nx % 4 != 0;
     const size_t smem = sizeof(SweepShared<R, T>) + (seam ? 9 * 32 * sizeof(Raw4<R>) : 0);
     auto kernel = seam ? sweep_kernel<PREC, KIND, false, T, true> : sweep_kernel<PREC, KIND, false, T, false>;
-    if constexpr (PREC == SMRT_PREC_F16 || PREC == SMRT_PREC_BF16) {
+    if constexpr (PREC == SMRT_PREC_F16) {
+        if (hp.rounding == SMRT_ROUND_STOCHASTIC) return cudaErrorInvalidValue;   // one update per launch is faster
+    }
+    if constexpr (PREC == SMRT_PREC_BF16) {
         if (hp.rounding == SMRT_ROUND_STOCHASTIC)
             kernel = seam ? sweep_kernel<PREC, KIND, true, T, true> : sweep_kernel<PREC, KIND, true, T, false>;
     }

@@ -285,11 +285,8 @@ __device__ __forceinline__ void sweep(const typename Prec<PREC>::R *__restrict__
             }
             #pragma unroll
             for (int a = 0; a < 9; ++a) {
-                const R v[4] = {P::to_r_sr(f2_lo(g[0][a]), sr_pop_bits(nh[0], a)),
-                                P::to_r_sr(f2_hi(g[0][a]), sr_pop_bits(nh[1], a)),
-                                P::to_r_sr(f2_lo(g[1][a]), sr_pop_bits(nh[2], a)),
-                                P::to_r_sr(f2_hi(g[1][a]), sr_pop_bits(nh[3], a))};
-                f[a].set(v);
+                f[a].x = P::to_r2_sr(f2_lo(g[0][a]), f2_hi(g[0][a]), sr_pop_bits(nh[0], a), sr_pop_bits(nh[1], a));
+                f[a].y = P::to_r2_sr(f2_lo(g[1][a]), f2_hi(g[1][a]), sr_pop_bits(nh[2], a), sr_pop_bits(nh[3], a));
             }
         } else {
             #pragma unroll

@@ -14,8 +14,8 @@ from paper_2409_01076_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
 
-# sweeps: one strip that a row fills, several, ragged ones, short and long segments
-WIDE = [(128, 3000), (600, 601), (599, 640), (721, 720), (1201, 500), (2047, 331)]
+# sweeps: the narrowest, one strip that a row fills, several, ragged ones, short and long segments
+WIDE = [(9, 41001), (30, 12100), (128, 3000), (600, 601), (599, 640), (721, 720), (1201, 500), (2047, 331)]
 # tiles: smallest, ragged, every plan of the rule
 SMALL = [(8, 8), (9, 11), (64, 64), (65, 31), (123, 130), (241, 9), (361, 70), (300, 301), (470, 430)]
 FLOWS = {"cavity": W.CAVITY, "periodic": W.ALL_PERIODIC, "couette": W.COUETTE,
@@ -50,6 +50,31 @@ def test_one_call_equals_single_updates(size, flow, prec, kind, rounding):
         got, t = fields(*size, FLOWS[flow], prec, kind, rounding, calls)
         assert t == 13
         assert np.array_equal(one, got), (calls, np.abs(one - got).max())
+
+
+@pytest.mark.parametrize("size", [(4096, 4096), (4099, 4097), (4095, 4096)])    # the last one is below the rule
+@pytest.mark.parametrize("flow", ["cavity", "periodic"])
+def test_stochastic_rounding_at_the_size_that_takes_passes(size, flow):
+    import torch
+    nx, ny = size
+    x = torch.arange(nx, device="cuda", dtype=torch.float64)
+    y = torch.arange(ny, device="cuda", dtype=torch.float64)[:, None]
+    rho = 1.0 + 0.01 * torch.sin(0.37 * x) * torch.cos(0.11 * y)
+    u = torch.stack([0.05 * torch.sin(0.05 * x) * torch.cos(0.3 * y), 0.05 * torch.cos(0.2 * x + 0.07 * y)])
+    out = []
+    for calls in ([1] * 5, [5], [2, 3]):
+        h = make(nx, ny, 0.6, 0.1, FLOWS[flow], "bf16", "ab", "smrt")
+        S.smrt_set_option(h, S.SMRT_OPT_ROUNDING, S.SMRT_ROUND_STOCHASTIC)
+        S.smrt_init_macros(h, rho, u)
+        for n in calls:
+            S.smrt_step(h, n)
+        r, v = torch.empty_like(rho), torch.empty_like(u)
+        S.smrt_macros(h, r, v)
+        S.smrt_sync(h)
+        S.smrt_destroy(h)
+        out.append((r, v))
+    for r, v in out[1:]:
+        assert torch.equal(r, out[0][0]) and torch.equal(v, out[0][1])
 
 
 @pytest.mark.parametrize("prec", ["f64", "f32", "f16"])
