@@ -585,14 +585,14 @@ class UNet:
         t = self.torch
         rec = self._predict_rec
         if rec is not None and rec[0] == key:
-            rec[2].copy_(x)
+            rec[2].copy_(x.detach())
             rec[1].replay()
             return rec[3].clone()
         if self._predict_last != key:
             self._predict_last = key
             return self.forward(x, None)
         self._predict_rec = rec = None
-        xs = x.clone()
+        xs = x.detach().clone()
         side = t.cuda.Stream()
         side.wait_stream(t.cuda.current_stream())
         g = t.cuda.CUDAGraph()
