@@ -241,9 +241,10 @@ SMRT_API void smrt_destroy(smrt_t *h);
 
 /* ---- batches of independent lattices ------------------------------------------
  * Many lattices ("cavities") of uneven size and relaxation time, advanced by the
- * same update as smrt_step (bit for bit: the same per-block kernel code) in one
- * launch per step: a persistent work-list kernel walks the step blocks of every
- * active lattice.  Lattice k has nx[k] x ny[k] nodes, tau[k], u_lid[k]; all share
+ * same update as smrt_step (bit for bit: the same per-block kernel code) in
+ * launches that cover every active lattice: a persistent work-list kernel walks
+ * their step blocks, or one block per row segment makes two or three updates.
+ * Lattice k has nx[k] x ny[k] nodes, tau[k], u_lid[k]; all share
  * bc_flags, the collision kind (SMRT or SRT), the precision (F32 or F64) and the
  * layout.  Each lattice starts at f = f^eq(1, 0), t = 0.  Lattices retire
  * (stop advancing) in smrt_batch_run when converged, capped or diverged.
@@ -280,8 +281,10 @@ SMRT_API int smrt_batch_autotune(smrt_batch_t *b, int steps, int *choice);
  * The lattices' state is untouched: every shape computes the same bits. */
 SMRT_API int smrt_batch_set_shape(smrt_batch_t *b, int shape);
 
-/* n >= 0 updates of every active lattice (one work-list launch each); waits,
- * then marks lattices whose divergence word is set as SMRT_BATCH_DIVERGED. */
+/* n >= 0 updates of every active lattice (one work-list launch each; with FP32
+ * storage, the AB layout and lattices of at least 8 x 8, launches of two or three
+ * updates where n allows, whatever the tile shape); waits, then marks lattices
+ * whose divergence word is set as SMRT_BATCH_DIVERGED. */
 SMRT_API int smrt_batch_step(smrt_batch_t *b, long long n);
 
 /* Runs until no lattice is active: replays a CUDA graph of check_every updates

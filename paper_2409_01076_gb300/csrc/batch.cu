@@ -1,7 +1,8 @@
 // batch.cu -- many independent lattices ("cavities") of uneven size and
 // viscosity advanced together (the C ABI smrt_batch_* of include/smrt.h).
 //
-// Every step is ONE launch of a persistent work-list kernel: a fixed grid
+// Float two-buffer batches take two or three updates per launch, one block per lattice, strip and row segment
+// (batch_sweep_kernel).  Every other step is ONE launch of a persistent work-list kernel: a fixed grid
 // (SM count x resident blocks) walks the concatenated step-block lists of the
 // active lattices; each block runs the single-lattice step_block (the same
 // code, hence the same bits, as smrt_step) on its lattice's own slice of one
