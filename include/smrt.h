@@ -283,7 +283,8 @@ SMRT_API int smrt_batch_set_shape(smrt_batch_t *b, int shape);
 
 /* n >= 0 updates of every active lattice (one work-list launch each; with FP32
  * storage, the AB layout and lattices of at least 8 x 8, launches of two or three
- * updates where n allows, whatever the tile shape); waits, then marks lattices
+ * updates where n allows and many narrow lattices do not make that slower,
+ * whatever the tile shape); waits, then marks lattices
  * whose divergence word is set as SMRT_BATCH_DIVERGED. */
 SMRT_API int smrt_batch_step(smrt_batch_t *b, long long n);
 

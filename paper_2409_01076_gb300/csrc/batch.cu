@@ -20,6 +20,7 @@
 
 #include <new>
 #include <string>
+#include <algorithm>
 #include <vector>
 
 #include "kernels.cuh"
@@ -760,6 +761,23 @@ int check_index(smrt_batch_t *b, int k)
     return SMRT_OK;
 }
 
+// Whether sweeps of `rows` rows (`items` of them) beat one update per launch, in us per update.  A sweep's warp
+// takes 128 columns whatever the lattice has, the step blocks of a lattice up to 64 wide only its own, so many
+// narrow lattices are better off one by one.  A row of single updates was measured to take 0.6 ns (16-32 wide),
+// 0.82 ns (40-64), 1.35-2.4 ns (72-150) and 0.0115 ns a column beyond, at least the 6.2 us of a launch; sweeps
+// took 1.1-1.5 times sweep_rows' model in batches of narrow lattices, and 1.25 separates the pairs measured
+// (MLUPS, one by one / sweeps): 3,000 lattices of 32^2 56.3k / 40.5k, of 48^2 59.7k / 62.9k, of 64^2 78.4k / 85.5k, of 72^2 53.4k / 96.5k;
+// 300 of 32^2 35.9k / 18.5k, of 64^2 71.3k / 47.7k, of 72^2 44.2k / 54.5k, of 150^2 64.0k / 102.3k; 8 of 64^2
+// 5.3k / 7.5k; 2,000 of 256^2 88.8k / 156.3k.  The rate of wide lattices is set low: there sweeps always won.
+bool sweeps_pay(const std::vector<Lat> &lat, int rows, long long items)
+{
+    double single = 0.0;
+    for (const Lat &L : lat)
+        single += 1e-3 * L.ny * (L.nx <= 32 ? 0.6 : L.nx <= 64 ? 0.82 : std::max(1.5, 0.016 * L.nx));
+    const double one = std::max(0.685, 0.35 + 0.30 * (double)items / 608.0);
+    return 1.25 * (2.0 + (rows + 2) * one) < std::max(6.2, single);
+}
+
 } // namespace
 
 extern "C" {
@@ -845,6 +863,7 @@ int smrt_batch_create(int count, const int *nx, const int *ny, const double *tau
             b->sweep_rows = smrt::sweep_rows(strips.data(), rows.data(), count, 3);
             for (int k = 0; k < count; ++k)
                 b->max_items += (long long)strips[k] * ((rows[k] + b->sweep_rows - 1) / b->sweep_rows);
+            if (!sweeps_pay(b->lat, b->sweep_rows, b->max_items)) b->sweep_rows = b->max_items = 0;
         }
     }
     if (b->max_work >= (1LL << 31) || b->max_items >= (1LL << 31)) {

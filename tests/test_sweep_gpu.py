@@ -91,3 +91,23 @@ def test_divergence_is_reported(prec, size, node):
         S.smrt_step(h, 3)
     assert e.value.status == S.SMRT_ERR_DIVERGED
     S.smrt_destroy(h)
+
+
+# many lattices of one narrow width take one update per launch, few or wider ones passes
+@pytest.mark.parametrize("count,nx,ny", [(300, 8, 8), (300, 32, 19), (300, 64, 33), (300, 72, 33), (3, 64, 33), (1, 8, 8)])
+@pytest.mark.parametrize("kind", ["smrt", "srt"])
+def test_batch_of_one_width_equals_single_lattices(count, nx, ny, kind):
+    tau = [0.6 + 0.3 * k / count for k in range(count)]
+    b = S.smrt_batch_create([nx] * count, [ny] * count, tau, [0.08] * count, W.CAVITY, S.SMRT_PREC_F32, S.SMRT_LAYOUT_AB,
+                            {"smrt": S.SMRT_COLLISION_SMRT, "srt": S.SMRT_COLLISION_SRT}[kind])
+    for n in (1, 5, 8):
+        S.smrt_batch_step(b, n)
+    for k in {0, count // 2, count - 1}:
+        h = make(nx, ny, tau[k], 0.08, W.CAVITY, "f32", "ab", kind)
+        for _ in range(14):
+            S.smrt_step(h, 1)
+        f = np.empty((9, ny, nx))
+        S.smrt_batch_get_f(b, k, f)
+        assert np.array_equal(get_f(h), f), k
+        S.smrt_destroy(h)
+    S.smrt_batch_destroy(b)
