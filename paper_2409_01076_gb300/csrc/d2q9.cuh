@@ -48,7 +48,9 @@ static_assert(ex(opp(6)) == -ex(6) && ey(opp(6)) == -ey(6), "opp");
 // ---- launches that follow one another -------------------------------------------
 // An update kernel may be launched before the one in front of it has quite ended (programmatic dependent launch):
 // its blocks come up while their predecessor's last ones drain, and wait for it to be complete, with its writes
-// visible, before they touch the state.  What overlaps is launch latency alone, 0.5-2 us per launch (us per update,
+// visible, before they touch the state.  What the predecessor writes is therefore not constant over the kernel's
+// lifetime: such a kernel must not take it as a __restrict__ parameter, which would allow non-coherent loads and
+// loads moved in front of the wait.  What overlaps is launch latency alone, 0.5-2 us per launch (us per update,
 // before -> after: 64^2 f64 3.8 -> 3.3, 256^2 f64 10.3 -> 8.8, 256^2 f32 in place 6.2 -> 4.1, 1021 x 509 f32
 // 6.2 -> 5.4, 1024^2 f32 10.3 -> 9.7).  Letting the successor up as soon as all blocks have started
 // (griddepcontrol.launch_dependents) was worse: its waiting blocks crowd the running ones (256^2 f64 20.7).

@@ -23,7 +23,7 @@ struct TileSalts {
 
 template <int PREC, int KIND, bool SR>
 __global__ void __launch_bounds__(512)
-tile_kernel(const typename Prec<PREC>::R *__restrict__ src, typename Prec<PREC>::R *__restrict__ dst,
+tile_kernel(const typename Prec<PREC>::R *src, typename Prec<PREC>::R *dst,
             const Params<typename Prec<PREC>::C> p, const TileSalts salt, int W, int H, int T, int tiles_x)
 {
     using P = Prec<PREC>;
