@@ -72,7 +72,9 @@ inline cudaError_t launch_following(void (*kernel)(P...), unsigned blocks, unsig
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    if (e != cudaSuccess) cudaGetLastError();        // told here: not to be found again by the next launch
+    return e;
 }
 
 // ---- storage formats ----------------------------------------------------------
