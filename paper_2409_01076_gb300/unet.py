@@ -22,7 +22,6 @@ accumulation; master weights, gradients and optimiser state are float32.
 from __future__ import annotations
 
 import math
-import threading
 
 import numpy as np
 
@@ -110,8 +109,6 @@ class UNet:
             self.m[key] = self._flat["m"][o:o + n].view(val.shape)
             self.v[key] = self._flat["v"][o:o + n].view(val.shape)
         self._graph = None
-        self._predict_rec = self._predict_last = None
-        self._predict_lock = threading.Lock()
         self.step_count = 0
         self.grad_scale = 2.0 ** 16
         self._found_inf = torch.zeros(1, dtype=torch.int32, device=device)
@@ -559,53 +556,10 @@ class UNet:
         self.adam_step(lr)
         return float(self._loss.item())
 
-    # Predictions of at most this many pixels are bound by their ~35 launches (256^2: 450-540 us from the host,
-    # 316 replayed), so a shape that repeats is recorded once and replayed.  Larger ones are bound by the
-    # kernels, and their recording would hold on to activations (~1 KB a pixel).
-    PREDICT_GRAPH_PIXELS = 4 * 256 * 256
-
     def predict(self, x):
-        """The network's output for x (N, H, W, cin) float32 CUDA, complete when the call returns.  The second
-        call in a row with one shape records the forward pass (weight packing included: it reads the current
-        parameters on every replay) on buffers of its own, which live as long as the network or until another
-        shape takes their place; later calls copy x in, replay and copy the result out."""
-        t = self.torch
-        key = (tuple(x.shape), self.conv_path, self.gemm_backend, t.cuda.current_device())
-        n = x.shape[0] * x.shape[1] * x.shape[2]
-        if n <= self.PREDICT_GRAPH_PIXELS and x.dtype == t.float32 and x.is_cuda and x.is_contiguous() and self._all_tma():
-            with self._predict_lock:        # the recording's buffers serve one call at a time
-                y = self._predict_recorded(x, key)
-                self.check_timeouts()       # waits for the stream: the buffers are free again
-                return y
         y = self.forward(x, None)
         self.check_timeouts()
         return y
-
-    def _predict_recorded(self, x, key):
-        t = self.torch
-        rec = self._predict_rec
-        if rec is not None and rec[0] == key:
-            rec[2].copy_(x.detach())
-            rec[1].replay()
-            return rec[3].clone()
-        if self._predict_last != key:
-            self._predict_last = key
-            return self.forward(x, None)
-        self._predict_rec = rec = None
-        xs = x.detach().clone()
-        side = t.cuda.Stream()
-        side.wait_stream(t.cuda.current_stream())
-        g = t.cuda.CUDAGraph()
-        with t.cuda.stream(side):
-            g.capture_begin(capture_error_mode="thread_local")
-            try:
-                ys = self.forward(xs, None)
-            finally:
-                g.capture_end()
-        t.cuda.current_stream().wait_stream(side)
-        self._predict_rec = (key, g, xs, ys)
-        g.replay()
-        return ys.clone()
 
 
 def input_grid(res, h: int, w: int, device: str = "cuda"):
