@@ -548,8 +548,12 @@ init_macros_kernel(typename Prec<PREC>::R *state, const double *rho, const doubl
     }
 }
 
+__device__ __forceinline__ unsigned upper_abs(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+
 // Moments of Eq. (fea-0) in double from the canonical offsets: 28 double operations.  1/rho by recip_d; one
-// correction step makes u the rounded quotient again.
+// correction step makes u the rounded quotient again.  Where recip_d is no reciprocal (rho zero, infinite, NaN or
+// at the ends of the range) or a product has overflowed, u is the quotient itself: a node without mass has the
+// infinite velocity that the division gives.
 __device__ __forceinline__ void moments_d(const double g[9], double &rho, double &ux, double &uy)
 {
     const double drho = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
@@ -557,6 +561,12 @@ __device__ __forceinline__ void moments_d(const double g[9], double &rho, double
     const double jx = (g[1] - g[3]) + (d57 - d68), jy = (g[2] - g[4]) + (d57 + d68);
     rho = 1.0 + drho;
     const double inv = recip_d(rho), qx = jx * inv, qy = jy * inv;
+    if (upper_abs(rho) - 0x00300000u >= 0x7f800000u || upper_abs(qx) >= 0x7ff00000u ||      // not 2^-1020 <= |rho| < 2^1020
+        upper_abs(qy) >= 0x7ff00000u) {
+        ux = jx / rho;
+        uy = jy / rho;
+        return;
+    }
     ux = fma(fma(-qx, rho, jx), inv, qx);
     uy = fma(fma(-qy, rho, jy), inv, qy);
 }
