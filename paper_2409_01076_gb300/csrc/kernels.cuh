@@ -464,35 +464,59 @@ __global__ void set_f_kernel(typename Prec<PREC>::R *state, const double *f, int
 // One population of f^eq(rho, u) (Eq. feq-full) as an offset, stored through the pull map.
 // Float arithmetic for the 32- and 16-bit formats (their stored value has at most 24
 // significant bits); the weight product is rounded as for an exact weight.
-template <int PREC, int MODE, int A>
+template <int PREC, int MODE, bool INNER, int A = 0>
 __device__ __forceinline__ void init_store_f(typename Prec<PREC>::R *state, const Params<float> &p, int i, int j,
-                                             bool inner, float drho, float d, float ux, float uy, float uu)
+                                             float drho, float d, float ux, float uy, float uu)
 {
     using P = Prec<PREC>;
     const float eu = float(ex(A)) * ux + float(ey(A)) * uy;
     float g = WeightMul<float>::template mul<A>(drho + d * (3.0f * eu + 4.5f * eu * eu - 1.5f * uu));
-    if (inner) {
+    if constexpr (INNER) {
         state[inner_at<MODE>(p, A, i, j)] = P::to_r(g);
-        return;
+    } else {
+        const Loc L = pull_loc<MODE>(p, A, i, j);
+        if (L.side >= 0) g -= p.corr[L.side][A];
+        state[at(p.plane, p.pitch, L.plane, L.j, L.i)] = P::to_r(g);
     }
-    const Loc L = pull_loc<MODE>(p, A, i, j);
-    if (L.side >= 0) g -= p.corr[L.side][A];
-    state[at(p.plane, p.pitch, L.plane, L.j, L.i)] = P::to_r(g);
+    if constexpr (A < 8) init_store_f<PREC, MODE, INNER, A + 1>(state, p, i, j, drho, d, ux, uy, uu);
 }
 
-// Blocks of the field kernels below: 256 consecutive nodes of one row, so that a node's row and column
-// need no division per thread.
+// Blocks of the field kernels below: 256 consecutive nodes of one row, so that a node's row and column need no
+// division per thread, or `pack` whole rows of a lattice that is narrower and has more rows than 8 blocks per SM
+// take one by one (a shorter lattice's rows stay apart, each on an SM of its own).  Measured, us, one row per
+// block -> packed: FP32 fields out of 8 x 500,000 443 -> 126, of 16 x 250,000 229 -> 93; FP32 fields into 8 x 500,000
+// 415 -> 90, 16 x 250,000 215 -> 70; FP64 out 1,051 -> 269 and 531 -> 267.
 constexpr int kFieldBX = 256;
+inline int field_pack(int rows, int nx)
+{
+    const int most = nx < kFieldBX ? kFieldBX / nx : 1, spare = rows / (8 * 152);
+    return spare < 1 ? 1 : (spare < most ? spare : most);
+}
 inline unsigned field_blocks(int rows, int nx)
 {
-    return (unsigned)((long long)rows * ((nx + kFieldBX - 1) / kFieldBX));
+    const int pack = field_pack(rows, nx);
+    return (unsigned)((((long long)rows + pack - 1) / pack) * ((nx + kFieldBX - 1) / kFieldBX));
 }
-__device__ __forceinline__ bool field_node(int nx, int &r, int &i)
+__device__ __forceinline__ bool field_node(int rows, int nx, int pack, int &r, int &i)
 {
+    if (pack > 1) {
+        const unsigned k = threadIdx.x / (unsigned)nx;
+        r = (int)(blockIdx.x * (unsigned)pack + k);
+        i = (int)(threadIdx.x - k * (unsigned)nx);
+        return (int)k < pack && r < rows;
+    }
     const unsigned per_row = (unsigned)(nx + kFieldBX - 1) / kFieldBX;
     r = (int)(blockIdx.x / per_row);
     i = (int)((blockIdx.x - (unsigned)r * per_row) * kFieldBX + threadIdx.x);
     return i < nx;
+}
+
+// Whether all of the warp's nodes have their nine source nodes inside the lattice: one path per warp, not both where
+// it holds a node at a side (FP32 fields into 64 x 62,500: 84 -> 68 us; one branch for the nine stores 2048^2 52 -> 48).
+template <class C>
+__device__ __forceinline__ bool warp_inner(const Params<C> &p, int i, int j)
+{
+    return __all_sync(__activemask(), i >= 1 && i + 1 < p.nx && j >= 1 && j + 1 < p.ny);
 }
 
 // f = f^eq(rho, u) (Eq. feq-full), written as offsets through the pull map;
@@ -502,11 +526,11 @@ __device__ __forceinline__ bool field_node(int nx, int &r, int &i)
 template <int PREC, int MODE>
 __global__ void __launch_bounds__(kFieldBX)
 init_macros_kernel(typename Prec<PREC>::R *state, const double *rho, const double *u,
-                   int row0, int rows, const Params<typename Prec<PREC>::C> p)
+                   int row0, int rows, int pack, const Params<typename Prec<PREC>::C> p)
 {
     using P = Prec<PREC>;
     int r, i;
-    if (!field_node(p.nx, r, i)) return;
+    if (!field_node(rows, p.nx, pack, r, i)) return;
     const int j = row0 + r;
     const size_t q = (size_t)r * p.nx + i;
     double d = 1.0, ux = 0.0, uy = 0.0;           // rho == NULL: the resting state
@@ -535,16 +559,8 @@ init_macros_kernel(typename Prec<PREC>::R *state, const double *rho, const doubl
     } else {
         const float drho = (float)(d - 1.0), df = (float)d, fx = (float)ux, fy = (float)uy;
         const float uu = fx * fx + fy * fy;
-        const bool inner = i >= 1 && i + 1 < p.nx && j >= 1 && j + 1 < p.ny;
-        init_store_f<PREC, MODE, 0>(state, p, i, j, inner, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 1>(state, p, i, j, inner, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 2>(state, p, i, j, inner, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 3>(state, p, i, j, inner, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 4>(state, p, i, j, inner, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 5>(state, p, i, j, inner, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 6>(state, p, i, j, inner, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 7>(state, p, i, j, inner, drho, df, fx, fy, uu);
-        init_store_f<PREC, MODE, 8>(state, p, i, j, inner, drho, df, fx, fy, uu);
+        if (warp_inner(p, i, j)) init_store_f<PREC, MODE, true>(state, p, i, j, drho, df, fx, fy, uu);
+        else init_store_f<PREC, MODE, false>(state, p, i, j, drho, df, fx, fy, uu);
     }
 }
 
@@ -648,16 +664,18 @@ __device__ __forceinline__ void moments_any(const float g[9], double &rho, doubl
     moments_f(g, rho, ux, uy);
 }
 
+// (Eight blocks per SM in float: at 36 registers a thread six fit, and rows of 200 nodes took 107 us instead of 84.)
 template <int PREC, int MODE>
-__global__ void __launch_bounds__(kFieldBX)
-macros_kernel(const typename Prec<PREC>::R *state, double *rho, double *u, int row0, int rows,
+__global__ void __launch_bounds__(kFieldBX, PREC == SMRT_PREC_F64 ? 6 : 8)
+macros_kernel(const typename Prec<PREC>::R *state, double *rho, double *u, int row0, int rows, int pack,
               const Params<typename Prec<PREC>::C> p)
 {
     int r, i;
-    if (!field_node(p.nx, r, i)) return;
+    if (!field_node(rows, p.nx, pack, r, i)) return;
     const int j = row0 + r;
     typename Prec<PREC>::C g[9];
-    if (i >= 1 && i + 1 < p.nx && j >= 1 && j + 1 < p.ny) pull_inner<PREC, MODE>(state, p, i, j, g);
+    // (below 8 columns most nodes are at a side, and a warp would take both paths: 4 x 1 M, 235 us against 194)
+    if (p.nx >= 8 && i >= 1 && i + 1 < p.nx && j >= 1 && j + 1 < p.ny) pull_inner<PREC, MODE>(state, p, i, j, g);
     else pull_canonical<PREC, MODE>(state, p, i, j, g);
     double rr, ux, uy;
     moments_any(g, rr, ux, uy);
@@ -1085,7 +1103,8 @@ cudaError_t launch_init_macros(int mode, void *state, const double *rho, const d
     const Params<typename P::C> p = make_params<typename P::C>(hp);
     if (rows <= 0) return cudaSuccess;
     const unsigned nb = field_blocks(rows, hp.nx);
-    SMRT_MODE_SWITCH(mode, (init_macros_kernel<PREC, M><<<nb, kFieldBX, 0, s>>>((typename P::R *)state, rho, u, row0, rows, p)));
+    const int pack = field_pack(rows, hp.nx);
+    SMRT_MODE_SWITCH(mode, (init_macros_kernel<PREC, M><<<nb, kFieldBX, 0, s>>>((typename P::R *)state, rho, u, row0, rows, pack, p)));
     return cudaGetLastError();
 }
 
@@ -1097,7 +1116,8 @@ cudaError_t launch_macros(int mode, const void *state, double *rho, double *u, i
     const Params<typename P::C> p = make_params<typename P::C>(hp);
     if (rows <= 0) return cudaSuccess;
     const unsigned nb = field_blocks(rows, hp.nx);
-    SMRT_MODE_SWITCH(mode, (macros_kernel<PREC, M><<<nb, kFieldBX, 0, s>>>((const typename P::R *)state, rho, u, row0, rows, p)));
+    const int pack = field_pack(rows, hp.nx);
+    SMRT_MODE_SWITCH(mode, (macros_kernel<PREC, M><<<nb, kFieldBX, 0, s>>>((const typename P::R *)state, rho, u, row0, rows, pack, p)));
     return cudaGetLastError();
 }
 
