@@ -302,9 +302,13 @@ conv1x1_small(const float *__restrict__ x, int P, int C, const float *__restrict
 // db[o] += sum_p dy[p][o].  Thread: one channel quad of every step-th pixel, so that neighbouring threads
 // read x and write dx side by side and a thread keeps 4 COUT sums (one pixel per thread kept 48 COUT, at
 // 8 warps per SM: 96 us at 16 x 256^2 x 32, whose bytes take 41; by quads: 57 us).  A block adds its sums in
-// shared memory and then into dw / db with one atomic per entry.  C <= 64; the block is a multiple of C / 4.
+// shared memory and then into dw / db with one atomic per entry.  That last sum, block after block onto one float,
+// is where the rounding errors of dw and db come from, so the blocks are large and few: one per SM (error of dw against
+// 64 bits 1.9e-7 there; with 8 blocks of 256 threads per SM 5.3e-7).  C <= 64; the block is a multiple of C / 4.
+template <int COUT> struct HeadBwd { static constexpr int BX = 1024, per_sm = 1; };
+template <> struct HeadBwd<1> { static constexpr int BX = 640, per_sm = 2; };       // fewer registers, more threads
 template <int COUT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(HeadBwd<COUT>::BX, HeadBwd<COUT>::per_sm)
 conv1x1_small_bwd(const float *__restrict__ dy, const float *__restrict__ x, int P, int C,
                   const float *__restrict__ w, float *__restrict__ dx, float *dw, float *db)
 {
@@ -322,6 +326,8 @@ conv1x1_small_bwd(const float *__restrict__ dy, const float *__restrict__ x, int
             wq[o][i] = w[o * C + 4 * q + i];
         }
     }
+    constexpr int kInFlight = COUT == 1 ? 4 : 2;
+    #pragma unroll kInFlight
     for (unsigned p = blockIdx.x * per_block + threadIdx.x / Q; p < (unsigned)P; p += gridDim.x * per_block) {
         float g[COUT];
         #pragma unroll
@@ -343,11 +349,23 @@ conv1x1_small_bwd(const float *__restrict__ dy, const float *__restrict__ x, int
         }
         if (dx) stv<4>(dx + (size_t)p * C + 4 * q, d);
     }
+    // a warp's lanes of one quad first (Q a power of two: whole warps), then one shared-memory atomic per warp and entry
+    const bool lanes = (Q & (Q - 1)) == 0;
+    const bool adds = !lanes || (threadIdx.x & 31) < Q;
+    auto warp_quad = [&](float v) {
+        if (lanes)
+            for (int o = 16; o >= Q; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    };
     #pragma unroll
     for (int o = 0; o < COUT; ++o) {
-        if (q == 0) atomicAdd(&sacc[COUT * C + o], gb[o]);
+        const float b = warp_quad(gb[o]);
+        if (adds && q == 0) atomicAdd(&sacc[COUT * C + o], b);
         #pragma unroll
-        for (int i = 0; i < 4; ++i) atomicAdd(&sacc[o * C + 4 * q + i], gw[o][i]);
+        for (int i = 0; i < 4; ++i) {
+            const float v = warp_quad(gw[o][i]);
+            if (adds) atomicAdd(&sacc[o * C + 4 * q + i], v);
+        }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < COUT * C; i += blockDim.x)
@@ -461,17 +479,23 @@ cudaError_t small_conv1x1(const float *x, long long P, int C, const float *w, co
     return cudaGetLastError();
 }
 
+template <int COUT>
+void launch_head_bwd(const float *dy, const float *x, long long P, int C, const float *w, float *dx, float *dw, float *db,
+                     cudaStream_t s)
+{
+    const int threads = HeadBwd<COUT>::BX / (C / 4) * (C / 4);
+    long long b = (P + 127) / 128;                      // few pixels: at least 128 to a block
+    if (b > 152LL * HeadBwd<COUT>::per_sm) b = 152LL * HeadBwd<COUT>::per_sm;
+    conv1x1_small_bwd<COUT><<<(unsigned)b, threads, 0, s>>>(dy, x, (int)P, C, w, dx, dw, db);
+}
+
 cudaError_t small_conv1x1_bwd(const float *dy, const float *x, long long P, int C, const float *w, int cout, float *dx,
                               float *dw, float *db, cudaStream_t s)
 {
-    const int threads = 256 / (C / 4) * (C / 4);
-    long long b = (P * (C / 4) + threads - 1) / threads;
-    if (b > 152LL * 8) b = 152LL * 8;
-    const unsigned blocks = (unsigned)(b < 1 ? 1 : b);
     switch (cout) {
-    case 1: conv1x1_small_bwd<1><<<blocks, threads, 0, s>>>(dy, x, (int)P, C, w, dx, dw, db); break;
-    case 2: conv1x1_small_bwd<2><<<blocks, threads, 0, s>>>(dy, x, (int)P, C, w, dx, dw, db); break;
-    default: conv1x1_small_bwd<3><<<blocks, threads, 0, s>>>(dy, x, (int)P, C, w, dx, dw, db); break;
+    case 1: launch_head_bwd<1>(dy, x, P, C, w, dx, dw, db, s); break;
+    case 2: launch_head_bwd<2>(dy, x, P, C, w, dx, dw, db, s); break;
+    default: launch_head_bwd<3>(dy, x, P, C, w, dx, dw, db, s); break;
     }
     return cudaGetLastError();
 }

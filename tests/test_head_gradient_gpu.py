@@ -1,0 +1,44 @@
+"""The head's weight and bias gradients keep their accuracy: sums over a million pixels in float32."""
+import pytest
+import torch
+
+from paper_2409_01076_gb300 import nn as K
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("P,C,cout", [(1, 8, 1), (300, 4, 3), (19457, 60, 2), (155649, 12, 3)])
+def test_ragged_sizes(P, C, cout):
+    g = torch.Generator(device="cuda").manual_seed(P)
+    w, x = torch.randn(cout, C, generator=g, device="cuda"), torch.randn(P, C, generator=g, device="cuda")
+    dy = torch.randn(P, cout, generator=g, device="cuda")
+    dx, dw, db = torch.empty_like(x), torch.ones(cout, C, device="cuda"), torch.ones(cout, device="cuda")
+    K.smrt_nn_conv1x1_small_bwd(dy, x, w, dx, dw, db)
+    for got, a, b, start in ((dx, dy, w, 0.0), (dw, dy.T, x, 1.0), (db, dy.T, torch.ones(P, 1, device="cuda"), 1.0)):
+        want, size = a.double() @ b.double() + start, a.double().abs() @ b.double().abs() + start
+        assert ((got.double().view_as(want) - want).abs() <= 1e-6 * size).all()    # each value of its own terms
+
+
+@pytest.mark.parametrize("P,C,cout", [(1048576, 32, 3), (1048576, 64, 1), (65536, 32, 3), (65536, 20, 2), (4096, 64, 2)])
+def test_error_is_that_of_few_partial_sums(P, C, cout):
+    """Adding B partial sums one after another onto a float loses about 2^-25 (B / 3)^(1/2) of the sum in the mean
+    square; with B at most 304 and at most P / 128, as one pixel per thread in blocks of 128 had it, that is 3.0e-7,
+    the sums below average out; twice that for the bias, whose few entries are a small sample.  (At 1,216 partial
+    sums it is 6e-7.)"""
+    g = torch.Generator(device="cuda").manual_seed(P + C)
+    w = torch.randn(cout, C, generator=g, device="cuda")
+    blocks = min(304, max(2, P / 128))
+    bound = 2.0 ** -25 * (blocks / 3) ** 0.5
+    worst, worst_b = [], []
+    for _ in range(6):
+        x = torch.nn.functional.silu(torch.randn(P, C, generator=g, device="cuda"))
+        dy = torch.randn(P, cout, generator=g, device="cuda") + 0.2
+        dx, dw, db = torch.empty_like(x), torch.zeros(cout, C, device="cuda"), torch.zeros(cout, device="cuda")
+        K.smrt_nn_conv1x1_small_bwd(dy, x, w, dx, dw, db)
+        rw, rb = dy.double().T @ x.double(), dy.double().sum(0)
+        worst.append(float((dw.double() - rw).norm() / rw.norm()))
+        worst_b.append(float((db.double() - rb).norm() / rb.norm()))
+        rx = dy.double() @ w.double()
+        assert (dx.double() - rx).abs().max() <= 1e-6 * rx.abs().max()
+    assert sorted(worst)[3] <= max(bound, 1.2e-7), worst
+    assert sorted(worst_b)[3] <= 2 * max(bound, 1.2e-7), worst_b
