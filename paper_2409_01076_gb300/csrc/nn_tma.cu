@@ -492,12 +492,15 @@ conv3_tma_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant_
 // each), then adds alpha D_t into gw[o][t*C + c] with float32 atomics.
 // TN = 32: all nine taps (288 columns).  An MMA of 128 x 32 x 16 reads 5 KB of shared memory for 16 clocks of
 // tensor work, and issues no faster than one of 128 x 64 x 16, so where cout is a multiple of 64, TN = 64: half
-// the MMAs, in two kinds of CTA that take taps 0-4 and 5-8 (320 and 256 of the 512 columns) and split the pixel
-// tiles 5 : 4.
+// the MMAs, in two kinds of CTA (320 of the 512 columns each) that take taps 0-3 and 5-8 of the same pixel tiles,
+// and tap 4 of the first and the second half of them.  A column sums as many tiles one after another as TN = 32 has
+// it, or half as many: that chain makes the error.  16 x 128^2, 64 -> 64: TN = 32 77 us and an error of 4.07e-6 of
+// the gradient's norm; TN = 64 50 us, 3.90e-6.  (Tiles dealt out 5 : 4 to taps 0-4 and 5-8: 48.5 us, but chains of
+// 25 and 31 tiles instead of 27 and an error of 4.24e-6.)
 template <int TN>
 __global__ void __launch_bounds__(128)
 conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmz, int H, int W,
-                   int C, int cout, int tiles_x, int tiles_y, int ntiles, int nbk, int split0, int per0, int per1,
+                   int C, int cout, int tiles_x, int tiles_y, int ntiles, int nbk, int split, int per,
                    int planes, int nstages, int stage_bytes, float alpha, float *gw, int ldg, int *err)
 {
     extern __shared__ unsigned char dyn_raw[];
@@ -509,11 +512,10 @@ conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constan
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int mb = blockIdx.x / nbk, nb = blockIdx.x % nbk;
-    // CTAs [0, split0) of a channel block take the first taps, the others the rest
-    const bool second = (int)blockIdx.y >= split0;
-    const int tap0 = second ? 5 : 0, tap1 = (TN == 64 && !second) ? 5 : 9;
-    const int per = second ? per1 : per0;
-    const int t_beg = ((int)blockIdx.y - (second ? split0 : 0)) * per;
+    // CTAs [0, split) of a channel block are of the first kind
+    const bool second = (int)blockIdx.y >= split;
+    const int tap0 = second ? 4 : 0, tap1 = TN == 64 ? tap0 + 5 : 9;
+    const int t_beg = ((int)blockIdx.y - (second ? split : 0)) * per;
     const int t_end = min(ntiles, t_beg + per);
     if (t_beg >= t_end) return;             // uniform over the CTA
     const int a_bytes = (planes * kPlane + 127) / 128 * 128;
@@ -522,6 +524,8 @@ conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constan
 
     const uint32_t tmem = setup<kCols>(&tmem_holder, full, empty, &done, nstages, &failed);
     const int n_it = t_end - t_beg;
+    // tap 4 in its CTA's tiles [mid0, mid1); the other taps in all of them
+    const int half = (n_it + 1) / 2, mid0 = second ? half : 0, mid1 = (TN == 64 && !second) ? half : n_it;
 
     if (warp == 0 && lane == 0) {
         asm volatile("prefetch.tensormap [%0];" :: "l"(reinterpret_cast<uint64_t>(&tmx)) : "memory");
@@ -546,13 +550,14 @@ conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constan
             const uint32_t st = base + (uint32_t)(s * stage_bytes);
             #pragma unroll 1
             for (int t = tap0; t < tap1; ++t) {
-                const int ky = t / 3, kx = t % 3;
+                if (t == 4 && (it < mid0 || it >= mid1)) continue;
+                const int ky = t / 3, kx = t % 3, it0 = t == 4 ? mid0 : 0;
                 #pragma unroll
                 for (int j = 0; j < kTileRows / 2; ++j) {        // K = 16 pixels: image rows 2j, 2j + 1
                     mma_f16(tmem + (uint32_t)((t - tap0) * TN),
                             desc(st + (uint32_t)(((2 * j + ky) * kHaloPx + kx) * 16), kHaloPx * 16, kPlane),
                             desc(st + (uint32_t)a_bytes + (uint32_t)(2 * j * 128), 128, kDzPlane),
-                            idesc<TN, true>(), (it > 0 || j > 0) ? 1u : 0u);
+                            idesc<TN, true>(), (it > it0 || j > 0) ? 1u : 0u);
                 }
             }
             commit(smem_u32(&empty[s]));
@@ -568,6 +573,7 @@ conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constan
         const int c = kWgPlanes * 8 * mb + warp * 32 + lane;
         #pragma unroll 1
         for (int t = tap0; t < tap1; ++t) {
+            if (t == 4 && mid0 >= mid1) continue;
             #pragma unroll 1
             for (int o0 = 0; o0 < TN; o0 += 32) {
                 uint32_t r[32];
@@ -1301,12 +1307,11 @@ extern "C" int smrt_nn_conv3_wgrad_tma(const void *xb, int N, int H, int W, int 
     const int mbk = (C + 8 * kWgPlanes - 1) / (8 * kWgPlanes), nbk = (cout + TN - 1) / TN;
     // one CTA per SM (each holds all 512 TMEM columns): split the pixel tiles to fill the SMs
     const int kinds = TN == 64 ? 2 : 1;
-    long long splits = sm_count() / (mbk * nbk);
-    if (splits < kinds) splits = kinds;
-    long long split0 = TN == 64 ? (5 * splits + 4) / 9 : splits, split1 = splits - split0;
-    if (split0 > ntiles) split0 = ntiles;
-    if (split1 > ntiles) split1 = ntiles;
-    const int per0 = (int)((ntiles + split0 - 1) / split0), per1 = split1 ? (int)((ntiles + split1 - 1) / split1) : 1;
+    long long split = sm_count() / (mbk * nbk * kinds);
+    if (split < 1) split = 1;
+    if (split > ntiles) split = ntiles;
+    const int per = (int)((ntiles + split - 1) / split);
+    split = (ntiles + per - 1) / per;
     const int a_bytes = (planes * kPlane + 127) / 128 * 128;
     const int stage = (a_bytes + TN / 8 * kDzPlane + 1023) / 1024 * 1024;
     const int a_reach = kWgPlanes * kPlane;         // the MMA's 128 rows read 16 planes from a stage start
@@ -1315,7 +1320,7 @@ extern "C" int smrt_nn_conv3_wgrad_tma(const void *xb, int N, int H, int W, int 
     while (nstages > 2 && need(nstages) + 1024 > 220 * 1024) --nstages;
     size_t smem = need(nstages) + 1024;
     if (smem < 120 * 1024) smem = 120 * 1024;       // keeps a second CTA (and its TMEM request) off the SM
-    if (smem > 220 * 1024 || mbk * nbk > 65535 || splits > 65535)
+    if (smem > 220 * 1024 || mbk * nbk > 65535 || split * kinds > 65535)
         return tma_fail(SMRT_ERR_ARG, "smrt_nn_conv3_wgrad_tma: sizes out of range (C %d cout %d)", C, cout);
     auto kernel = TN == 64 ? conv3_wgrad_kernel<64> : conv3_wgrad_kernel<32>;
     static bool attr_set[2] = {false, false};
@@ -1324,9 +1329,9 @@ extern "C" int smrt_nn_conv3_wgrad_tma(const void *xb, int N, int H, int W, int 
         if (e != cudaSuccess) return tma_fail(SMRT_ERR_CUDA, "smrt_nn_conv3_wgrad_tma: %s", cudaGetErrorString(e));
         attr_set[kinds - 1] = true;
     }
-    dim3 grid(mbk * nbk, (unsigned)(split0 + split1));
+    dim3 grid(mbk * nbk, (unsigned)(split * kinds));
     kernel<<<grid, 128, smem, (cudaStream_t)stream>>>(tmx, tmz, H, W, C, cout, tiles_x, tiles_y, (int)ntiles, nbk,
-                                                      (int)split0, per0, per1, planes, nstages, stage, alpha, gw, ldg,
+                                                      (int)split, per, planes, nstages, stage, alpha, gw, ldg,
                                                       err);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return tma_fail(SMRT_ERR_CUDA, "smrt_nn_conv3_wgrad_tma: %s", cudaGetErrorString(e));
