@@ -309,7 +309,9 @@ SMRT_API int smrt_batch_run(smrt_batch_t *b, double tol, long long check_every, 
  * last residual of smrt_batch_run (-1 before the first check), smrt_batch_state. */
 SMRT_API int smrt_batch_status(const smrt_batch_t *b, long long *steps, double *residual, int *state);
 
-/* Canonical f(t) of lattice k as double[9][ny][nx] (host or device memory). */
+/* Canonical f(t) of lattice k as double[9][ny][nx] (host or device memory).  Arrays in host memory, here and
+ * in smrt_batch_macros and smrt_batch_init_macros, pass through device scratch, of which the batch keeps up to
+ * 64 MiB for the next call. */
 SMRT_API int smrt_batch_get_f(smrt_batch_t *b, int k, double *f);
 
 /* rho(t), u(t) of lattice k: double[ny][nx] and double[2][ny][nx], host or device. */

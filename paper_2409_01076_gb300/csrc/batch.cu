@@ -739,8 +739,18 @@ bool device_memory(const smrt_batch_t *b, const void *p)
            at.device == b->device && ((uintptr_t)p & 7u) == 0;
 }
 
-// At least n doubles of device scratch for fields in other memory, kept until the batch is destroyed (the
-// largest lattice's at most).  Every call that uses it waits for its stream before it returns.
+// At least n doubles of device scratch for fields in other memory.  Every call that uses it waits for its stream
+// before it returns, and then gives back scratch of more than 64 MiB (whose copies take far longer than its
+// allocation); smaller scratch stays until the batch is destroyed.
+constexpr size_t kStageKept = (size_t)64 << 20;
+void trim_stage(smrt_batch_t *b)
+{
+    if (b->stage_doubles * sizeof(double) <= kStageKept) return;
+    cudaFree(b->d_stage);
+    b->d_stage = nullptr;
+    b->stage_doubles = 0;
+}
+
 int ensure_stage(smrt_batch_t *b, size_t n, double **out)
 {
     if (b->stage_doubles < n) {
@@ -1141,6 +1151,7 @@ int smrt_batch_get_f(smrt_batch_t *b, int k, double *f)
     if (e == cudaSuccess && !dev)
         e = cudaMemcpyAsync(f, out, sizeof(double) * 9 * (size_t)L.nodes, cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    trim_stage(b);
     if (e != cudaSuccess) return bfail(b, SMRT_ERR_CUDA, "smrt_batch_get_f: %s", cudaGetErrorString(e));
     return SMRT_OK;
 }
@@ -1166,6 +1177,7 @@ int smrt_batch_macros(smrt_batch_t *b, int k, double *rho, double *u)
     if (e == cudaSuccess && !du)
         e = cudaMemcpyAsync(u, tu, sizeof(double) * 2 * (size_t)L.nodes, cudaMemcpyDefault, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    trim_stage(b);
     if (e != cudaSuccess) return bfail(b, SMRT_ERR_CUDA, "smrt_batch_macros: %s", cudaGetErrorString(e));
     return SMRT_OK;
 }
@@ -1198,6 +1210,7 @@ int smrt_batch_init_macros(smrt_batch_t *b, int k, const double *rho, const doub
     if (e == cudaSuccess)
         e = table(b->prec).init_macros(mode_of(b, L.t), lattice_state(b, k), sr, su, 0, L.ny, hp, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    trim_stage(b);
     if (e != cudaSuccess) return bfail(b, SMRT_ERR_CUDA, "smrt_batch_init_macros: %s", cudaGetErrorString(e));
     return SMRT_OK;
 }
