@@ -200,7 +200,7 @@ def kernel_source_hash():
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2409_01076_gb300", "csrc")
     for name in sorted(os.listdir(csrc)):
-        if name in ("d2q9.cuh", "kernels.cuh", "sweep.cuh") or (name.startswith("prec_") and name.endswith(".cu")):
+        if name in ("d2q9.cuh", "kernels.cuh", "sweep.cuh", "tile.cuh") or (name.startswith("prec_") and name.endswith(".cu")):
             with open(os.path.join(csrc, name), "rb") as fh:
                 h.update(name.encode() + b"\0" + fh.read())
     return h.hexdigest()[:16]
@@ -228,20 +228,6 @@ def committed_traffic(prec, layout, kind):
 
 
 # ---- the GPU arm ---------------------------------------------------------------------
-
-def update_launches(steps, nodes, prec, layout):
-    """Update kernels that smrt_step(steps) launches.  The two-buffer layout of a float format takes up to
-    three updates per pass over the state (the last ones by twos); a lattice of at most 600^2 nodes up to
-    eight, in tiles (then a lower bound); every other update is a launch of its own, and so is every one of
-    stochastic rounding but to BF16 from 4096^2 nodes on."""
-    if layout != "ab" or steps < 2:
-        return steps
-    if nodes <= 600 * 600:
-        return -(-steps // 8)
-    if prec in ("f64", "f16-sr") or (prec == "bf16-sr" and nodes < 4096 * 4096):
-        return steps
-    return -(-steps // 3)
-
 
 def make_handle(S, wl, prec, layout, kind, check=True):
     """prec: f64, f32, f16 or bf16, with "-sr" for stochastic rounding of the 16-bit formats."""
@@ -275,11 +261,11 @@ def run_variant(S, wl, rho_d, u_d, prec, layout, kind, steps, warmup, world):
     if wl["u0"] is not None:
         S.smrt_init_macros(h, rho_d, u_d)
     S.smrt_step(h, warmup)
+    launches, _ = S.smrt_step_plan(h, steps)
     ms = max_over_ranks(time_steps(S, h, steps, world), world)
     S.smrt_destroy(h)
     nodes = wl["nx"] * wl["ny"]
     mlups = nodes * steps / (ms * 1e-3) / 1e6
-    launches = update_launches(steps, nodes, prec, layout)
     return {"mlups": round(mlups, 1), "ms_per_step": round(ms / steps, 5),
             "hbm_gbs": round(BYTES_PER_NODE[prec.replace("-sr", "")] * nodes * launches / (ms * 1e-3) / 1e9, 1),
             "steps": steps, "launches": launches}
@@ -537,11 +523,11 @@ def gpu_arm(args):
         more += 60
     clk = clocks.stop()
     clk["untimed_updates"] = more
+    launches, kernel = S.smrt_step_plan(h, args.steps)
     S.smrt_destroy(h)
     ms = max_over_ranks(ms, world)
     sec = ms * 1e-3
     mlups = world * nodes * args.steps / sec / 1e6
-    launches = update_launches(args.steps, nodes, args.prec, args.layout)
     per_launch = sec / launches
     peak, peak_src = measured_hbm_peak()
     achieved = BYTES_PER_NODE[args.prec.replace("-sr", "")] * nodes / per_launch / 1e9
@@ -563,7 +549,7 @@ def gpu_arm(args):
                      "traffic": (round(traffic_per_node * nodes) if traffic_per_node else None),
                      "algorithmic_bytes_per_launch": BYTES_PER_NODE[args.prec.replace("-sr", "")] * nodes,
                      "updates_per_launch": round(args.steps / launches, 3),
-                     "kernel": "%s<%s,%s,%s>" % ("step_kernel" if launches == args.steps else "sweep_kernel", args.prec,
+                     "kernel": "%s<%s,%s,%s>" % (("step_kernel", "sweep_kernel", "tile_kernel")[kernel], args.prec,
                                                  args.kind, args.layout)},
         "gpu_launches": launches,
         "clocks": clk,

@@ -157,6 +157,16 @@ SMRT_API int smrt_set_stream(smrt_t *h, void *stream);
  * the flag clears on smrt_set_f / smrt_init_macros. */
 SMRT_API int smrt_step(smrt_t *h, long long n);
 
+/* What smrt_step(h, n) would launch: *launches update kernels, the first of them *kernel (enum
+ * smrt_kernel; the last may make fewer updates, a single one by SMRT_KERNEL_STEP).  Either may be NULL.
+ * Depends on sizes, precision, layout, rounding and n alone; touches no device. */
+enum smrt_kernel {
+    SMRT_KERNEL_STEP = 0,  /* one update                                                */
+    SMRT_KERNEL_SWEEP = 1, /* two or three updates in one pass over the state           */
+    SMRT_KERNEL_TILE = 2   /* two to eight updates of a small lattice, in shared memory */
+};
+SMRT_API int smrt_step_plan(smrt_t *h, long long n, long long *launches, int *kernel);
+
 /* Wait for the handle's stream; returns SMRT_ERR_DIVERGED if the divergence
  * flag is set (see smrt_step), else SMRT_OK or SMRT_ERR_CUDA. */
 SMRT_API int smrt_sync(smrt_t *h);

@@ -26,6 +26,7 @@ SMRT_ROUND_NEAREST, SMRT_ROUND_STOCHASTIC = 0, 1
 SMRT_COLLISION_SMRT, SMRT_COLLISION_SRT, SMRT_COLLISION_TWO_TAU = 0, 1, 2
 SMRT_LAYOUT_AB, SMRT_LAYOUT_AA = 0, 1
 SMRT_PREC_F64, SMRT_PREC_F32, SMRT_PREC_F16, SMRT_PREC_BF16 = 0, 1, 2, 3
+SMRT_KERNEL_STEP, SMRT_KERNEL_SWEEP, SMRT_KERNEL_TILE = 0, 1, 2
 
 _STATUS_NAMES = {0: "SMRT_OK", -1: "SMRT_ERR_ARG", -2: "SMRT_ERR_OOM", -3: "SMRT_ERR_CUDA",
                  -4: "SMRT_ERR_DIVERGED", -5: "SMRT_ERR_TIMEOUT", -6: "SMRT_ERR_STATE"}
@@ -111,6 +112,13 @@ def smrt_set_stream(h: Handle, stream=None) -> None:
 
 def smrt_step(h: Handle, n: int) -> None:
     _check(_lib.load().smrt_step(h, int(n)), h)
+
+
+def smrt_step_plan(h: Handle, n: int) -> tuple[int, int]:
+    """(update launches of smrt_step(h, n), the first one's SMRT_KERNEL_*); touches no device."""
+    launches, kernel = ctypes.c_longlong(), ctypes.c_int()
+    _check(_lib.load().smrt_step_plan(h, int(n), ctypes.byref(launches), ctypes.byref(kernel)), h)
+    return launches.value, kernel.value
 
 
 def smrt_sync(h: Handle) -> None:

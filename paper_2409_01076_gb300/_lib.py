@@ -24,6 +24,7 @@ SIGNATURES = [
     ("smrt_get_option", c_int, [c_void_p, c_int, ctypes.POINTER(c_double)]),
     ("smrt_set_stream", c_int, [c_void_p, c_void_p]),
     ("smrt_step", c_int, [c_void_p, c_longlong]),
+    ("smrt_step_plan", c_int, [c_void_p, c_longlong, ctypes.POINTER(c_longlong), ctypes.POINTER(c_int)]),
     ("smrt_sync", c_int, [c_void_p]),
     ("smrt_macros", c_int, [c_void_p, c_void_p, c_void_p]),
     ("smrt_residual", c_int, [c_void_p, c_void_p, c_void_p]),

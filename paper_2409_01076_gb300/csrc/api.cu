@@ -240,6 +240,28 @@ bool takes_sweeps(const smrt_t *h)
     return h->prec == SMRT_PREC_BF16 && (long long)h->nx * h->ny >= 4096LL * 4096;
 }
 
+// The next launch of smrt_step with `left` updates to go.
+struct Pass {
+    int kernel, updates;        // smrt_kernel
+    TilePlan tile;
+};
+
+Pass next_pass(const smrt_t *h, const TilePlan &tile, long long left)
+{
+    Pass p = {SMRT_KERNEL_STEP, 1, tile};
+    if (h->layout != SMRT_LAYOUT_AB || left < 2 || h->nx < 8 || h->ny < 8) return p;
+    if (tile.T) {
+        p.kernel = SMRT_KERNEL_TILE;
+        if (left < tile.T) p.tile = tile_shape(h->nx, h->ny, h->prec, tile.W, tile.H, (int)left);
+        p.updates = p.tile.T;
+    } else if (takes_sweeps(h)) {
+        // by threes, the rest by twos: a single update moves as much memory as a pass of three
+        p.kernel = SMRT_KERNEL_SWEEP;
+        p.updates = (left >= 5 || left == 3) ? 3 : 2;
+    }
+    return p;
+}
+
 int current_mode(const smrt_t *h)
 {
     if (h->layout == SMRT_LAYOUT_AB) return MODE_AB;
@@ -510,40 +532,34 @@ int smrt_step(smrt_t *h, long long n)
     CUDA_TRY(h, g.err);
     const KernelTable &T = table_for(h->prec);
     HostParams p = host_params(h);
-    const bool passes = h->layout == SMRT_LAYOUT_AB && n >= 2 && h->nx >= 8 && h->ny >= 8;
-    const TilePlan &tile = h->tile;
-    const bool sweeps = takes_sweeps(h);
-    for (long long s = 0; s < n; ++s) {
+    for (long long left = n; left > 0;) {
         cudaError_t e;
         p.t = h->t;
-        const long long left = n - s;
-        if (passes && left >= 2 && (tile.T || sweeps)) {
-            int k;
-            if (tile.T) {
-                TilePlan t = tile;
-                if (left < t.T) t = tile_shape(h->nx, h->ny, h->prec, t.W, t.H, (int)left);
-                k = t.T;
-                e = T.tile(h->collision, t, h->buf[h->cur], h->buf[1 - h->cur], p, h->stream);
-            } else {
-                // by threes, the rest by twos: a single update moves as much memory as a pass of three
-                k = (left >= 5 || left == 3) ? 3 : 2;
-                e = T.sweep(h->collision, k, h->buf[h->cur], h->buf[1 - h->cur], p, h->stream);
-            }
-            if (e == cudaSuccess) {
-                h->cur = 1 - h->cur;
-                h->t += k - 1;
-                s += k - 1;
-            }
-        } else if (h->layout == SMRT_LAYOUT_AB) {
-            e = T.step(h->collision, MODE_AB, h->buf[h->cur], h->buf[1 - h->cur], p, h->stream);
-            if (e == cudaSuccess) h->cur = 1 - h->cur;
-        } else {
-            e = T.step(h->collision, current_mode(h), h->buf[0], h->buf[0], p, h->stream);
-        }
+        const Pass pass = next_pass(h, h->tile, left);
+        void *src = h->buf[h->cur], *dst = h->layout == SMRT_LAYOUT_AB ? h->buf[1 - h->cur] : src;
+        if (pass.kernel == SMRT_KERNEL_TILE) e = T.tile(h->collision, pass.tile, src, dst, p, h->stream);
+        else if (pass.kernel == SMRT_KERNEL_SWEEP) e = T.sweep(h->collision, pass.updates, src, dst, p, h->stream);
+        else e = T.step(h->collision, current_mode(h), src, dst, p, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "step launch");
-        ++h->t;
+        if (h->layout == SMRT_LAYOUT_AB) h->cur = 1 - h->cur;
+        h->t += pass.updates;
+        left -= pass.updates;
     }
     if (h->check_div) return smrt_sync(h);
+    return SMRT_OK;
+}
+
+int smrt_step_plan(smrt_t *h, long long n, long long *launches, int *kernel)
+{
+    if (!h) return SMRT_ERR_ARG;
+    if (n < 0) return fail(h, SMRT_ERR_ARG, "smrt_step_plan: n must be >= 0 (got %lld)", n);
+    const TilePlan tile = tile_plan(h->nx, h->ny, h->prec);
+    const Pass first = next_pass(h, tile, n);
+    // all but the last few passes are like the first
+    long long count = n / first.updates > 2 ? n / first.updates - 2 : 0;
+    for (long long left = n - count * first.updates; left > 0; ++count) left -= next_pass(h, tile, left).updates;
+    if (launches) *launches = count;
+    if (kernel) *kernel = first.kernel;
     return SMRT_OK;
 }
 
