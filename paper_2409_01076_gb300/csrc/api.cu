@@ -179,14 +179,16 @@ TilePlan tile_shape(int nx, int ny, int prec, int W, int H, int updates)
 }
 
 // Whether and how the two-buffer layout takes several updates per launch in tiles (T == 0: it does not).
-// A launch costs 6.2-6.5 us of latency whatever it does.  Beyond that an update of `warps` warps per block
-// and `blocks` / 152 blocks per SM was measured to take (64^2 to 1024^2, 40 plans each)
-//   double: 0.52 us x the warps per SM (the double pipe), at least the 1.75 us of one warp's chain,
-//   float:  0.45 us + 0.06 us x the warps per SM.
-// The alternatives: one update per launch in double, 3.2 + 0.52 us per warp of the SM; sweeps of three in
-// float (sweep_rows' model).  Measured, us per update, before -> after: 64^2 f64 10.3 -> 3.6 (8 x 4, T = 4),
-// 128^2 f64 8.2 -> 5.2 (16 x 8, T = 4), 64^2 f32 6.2 -> 1.6 (8 x 4, T = 8), 256^2 f32 6.2 -> 2.8 (16 x 16,
-// T = 6).  256^2 f64 (12.3 against 10.3 one by one) and 512^2 f32 (7.2 against 6.2 by sweeps) stay out.
+// Float: a launch costs 6.2-6.5 us of latency whatever it does, an update of `warps` warps per block and
+// `blocks` / 152 blocks per SM 0.45 us + 0.06 us x the warps per SM; the alternative are sweeps of three
+// (sweep_rows' model).  Measured, us per update, one by one -> tiles: 64^2 6.2 -> 1.2 (8 x 4, T = 8), 256^2 6.2 -> 2.6
+// (16 x 16, T = 6); 512^2 (7.2 against 5.1 by sweeps) stays out.
+// Double: the launch 6.0 us, an update 0.48 us x the warps of the fullest SM (the double pipe), at least the
+// 1.6 us of one warp's chain; the alternative, one update per launch, 4.9 us or, where the pipe takes longer,
+// 1.75 + 0.53 us x the warps of the fullest SM (blocks of two).  Fitted to every plan at 21 sizes from 16^2 to 256^2 with
+// dependent launches on both sides; us per update, tiles / one by one: 64^2 3.3 / 4.7 (8 x 4, T = 4), 96^2 3.9 / 4.8,
+// 112^2 4.3 / 4.9 (24 x 4, T = 3), 16 x 1000 4.2 / 8.1 are taken; 144^2 6.0 / 5.3, 160^2 6.1 / 5.8, 256^2 11.9 / 8.9,
+// 500 x 40 6.0 / 5.7 are not.
 TilePlan tile_plan(int nx, int ny, int prec)
 {
     TilePlan best;
@@ -195,8 +197,9 @@ TilePlan tile_plan(int nx, int ny, int prec)
     const bool f64 = prec == SMRT_PREC_F64;
     double least;
     if (f64) {
-        least = 3.2 + 0.52 * ((double)nx * ny / 32.0 / 152.0);
-        if (least < 6.2) least = 6.2;
+        const long long blocks = (long long)ny * ((nx + 63) / 64);
+        least = 1.75 + 2 * 0.526 * (double)((blocks + 151) / 152);
+        if (least < 4.9) least = 4.9;
     } else {
         const int strips = nx <= 128 ? 1 : (nx + 111) / 120;
         least = 1e300;
@@ -205,20 +208,21 @@ TilePlan tile_plan(int nx, int ny, int prec)
             const double us = (6.0 + 3.0 * (rows + 2) * (one > 0.685 ? one : 0.685)) / 3.0;
             if (us < least) least = us;
         }
+        least *= 0.97;
     }
-    least *= 0.97;
     const int side[] = {4, 8, 16, 24, 32}, updates[] = {2, 3, 4, 6, 8};
     for (int T : updates)
         for (int W : side)
             for (int H : side) {
                 const TilePlan t = tile_shape(nx, ny, prec, W, H, T);
                 if (H > W || W + 2 * (T - 1) >= 64 || t.shared > 48 * 1024) continue;
-                const double per_sm = (double)t.tiles_x * t.tiles_y / 152.0;
-                double us = 6.4;
+                const long long tiles = (long long)t.tiles_x * t.tiles_y;
+                const double per_sm = f64 ? (double)((tiles + 151) / 152) : (double)tiles / 152.0;
+                double us = f64 ? 6.0 : 6.4;
                 for (int ring = T - 1; ring >= 0; --ring) {
                     const int warps = ((W + 2 * ring) * (H + 2 * ring) + 31) / 32;
                     const double w = warps * (per_sm > 1.0 ? per_sm : 1.0);
-                    us += f64 ? (0.52 * w > 1.75 ? 0.52 * w : 1.75) : 0.45 + 0.06 * w;
+                    us += f64 ? (0.48 * w > 1.6 ? 0.48 * w : 1.6) : 0.45 + 0.06 * w;
                 }
                 if (us / T < least) {
                     least = us / T;

@@ -88,3 +88,12 @@ def test_a_capture_records_as_many_launches(nx, ny, prec, layout, rounding):
         assert rt.cudaGraphDestroy(graph) == 0
     S.smrt_set_stream(h, None)
     S.smrt_destroy(h)
+
+
+@pytest.mark.parametrize("nx,ny,kernel", [
+    (16, 16, TILE), (64, 64, TILE), (96, 96, TILE), (112, 112, TILE), (128, 64, TILE), (16, 1000, TILE),
+    (144, 144, STEP), (192, 192, STEP), (256, 256, STEP), (500, 40, STEP), (40, 500, STEP), (300, 100, STEP)])
+def test_double_tiles_where_they_were_measured_faster(nx, ny, kernel):
+    """Tiles against one update per launch on 152 SMs, both measured: 64^2 3.3 / 4.7 us per update, 112^2 4.3 / 4.9,
+    16 x 1000 4.2 / 8.1; 144^2 6.0 / 5.3, 500 x 40 6.0 / 5.7."""
+    assert plan(nx, ny, "f64", 240)[1] == kernel
