@@ -235,13 +235,14 @@ TilePlan tile_plan(int nx, int ny, int prec)
 // Whether updates that no tiles take go by sweeps of three: always for float storage and for 16 bits rounded
 // to nearest.  Stochastic rounding is bound by its own arithmetic, and a sweep spends it on the halo too.
 // Measured, one update per launch against sweeps, MLUPS: FP16 138.3k / 136.0k at 8192^2, 130.7k / 123.5k at
-// 4096^2, 104.1k / 65.3k for a 1024^2 cavity, 60.9k / 38.3k at 512^2; BF16 172.0k / 205.7k at 8192^2, 163.4k /
-// 183.8k for a 4096^2 cavity, 121.7k / 92.6k for a 1024^2 cavity.
+// 4096^2, 104.1k / 65.3k for a 1024^2 cavity, 60.9k / 38.3k at 512^2; BF16, us per update of a cavity, 8.5 / 11.3 at
+// 1024^2, 15.9 / 20.2 at 1536^2, 30.8 / 28.2 at 2048^2, 44.4 / 43.6 at 2560^2, 61.0 / 57.6 at 3072^2, 102.6 / 91.1 at
+// 4096^2, 153.8 / 127.8 at 5000^2.
 bool takes_sweeps(const smrt_t *h)
 {
     if (h->prec == SMRT_PREC_F64) return false;
     if (h->prec == SMRT_PREC_F32 || h->rounding != SMRT_ROUND_STOCHASTIC) return true;
-    return h->prec == SMRT_PREC_BF16 && (long long)h->nx * h->ny >= 4096LL * 4096;
+    return h->prec == SMRT_PREC_BF16 && (long long)h->nx * h->ny >= 2048LL * 2048;
 }
 
 // The next launch of smrt_step with `left` updates to go.

@@ -97,3 +97,31 @@ def test_double_tiles_where_they_were_measured_faster(nx, ny, kernel):
     """Tiles against one update per launch on 152 SMs, both measured: 64^2 3.3 / 4.7 us per update, 112^2 4.3 / 4.9,
     16 x 1000 4.2 / 8.1; 144^2 6.0 / 5.3, 500 x 40 6.0 / 5.7."""
     assert plan(nx, ny, "f64", 240)[1] == kernel
+
+
+def test_bf16_stochastic_rounding_takes_passes_from_2048_squared():
+    """One per launch / passes: 15.9 / 20.2 us at 1536^2, 30.8 / 28.2 at 2048^2."""
+    sr = S.SMRT_ROUND_STOCHASTIC
+    assert plan(2048, 2048, "bf16", 60, rounding=sr) == (20, SWEEP)
+    assert plan(2048, 2047, "bf16", 60, rounding=sr) == (60, STEP)
+    assert plan(2048, 2047, "bf16", 60) == (20, SWEEP)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny", [(2048, 2048), (2049, 2051)])
+@pytest.mark.parametrize("flow", [W.CAVITY, W.ALL_PERIODIC], ids=["cavity", "periodic"])
+def test_bf16_stochastic_rounding_by_passes_is_the_same(nx, ny, flow):
+    import numpy as np
+    fields = []
+    for calls in ([1] * 5, [5], [2, 3]):
+        h = make(nx, ny, 0.6, 0.1, flow, "bf16")
+        S.smrt_set_option(h, S.SMRT_OPT_ROUNDING, S.SMRT_ROUND_STOCHASTIC)
+        S.smrt_init_macros(h, *W.random_macros(nx, ny, seed=5, u_amp=0.03))
+        for n in calls:
+            S.smrt_step(h, n)
+        rho, u = np.empty((ny, nx)), np.empty((2, ny, nx))
+        S.smrt_macros(h, rho, u)
+        S.smrt_destroy(h)
+        fields.append((rho, u))
+    for rho, u in fields[1:]:
+        assert np.array_equal(rho, fields[0][0]) and np.array_equal(u, fields[0][1])
