@@ -34,6 +34,7 @@
 // bounded by 1 s of %globaltimer: a wait that gives up sets *err and the CTA's failed flag, waits
 // once more with the same bound (so no copy or MMA is left in flight where avoidable), skips the
 // epilogue, and the CTA still releases its tensor memory.
+#include <algorithm>
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -492,16 +493,16 @@ conv3_tma_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant_
 // each), then adds alpha D_t into gw[o][t*C + c] with float32 atomics.
 // TN = 32: all nine taps (288 columns).  An MMA of 128 x 32 x 16 reads 5 KB of shared memory for 16 clocks of
 // tensor work, and issues no faster than one of 128 x 64 x 16, so where cout is a multiple of 64, TN = 64: half
-// the MMAs, in two kinds of CTA (320 of the 512 columns each) that take taps 0-3 and 5-8 of the same pixel tiles,
-// and tap 4 of the first and the second half of them.  A column sums as many tiles one after another as TN = 32 has
-// it, or half as many: that chain makes the error.  16 x 128^2, 64 -> 64: TN = 32 77 us and an error of 4.07e-6 of
-// the gradient's norm; TN = 64 50 us, 3.90e-6.  (Tiles dealt out 5 : 4 to taps 0-4 and 5-8: 48.5 us, but chains of
-// 25 and 31 tiles instead of 27 and an error of 4.24e-6.)
+// the MMAs, in two kinds of CTA (320 of the 512 columns at most).  They take taps 0-4 and 5-8 and deal out the pixel
+// tiles 5 : 4 among them, as long as no column sums more tiles one after another than TN = 32 would: that chain makes
+// the error.  Where it would, both kinds take the same tiles (`share`), taps 0-3 and 5-8, and tap 4 of the first and
+// the second half of them.  16 x 128^2, 64 -> 64: TN = 32 77 us and an error of 4.07e-6 of the gradient's norm; shared
+// 50 us, 3.90e-6 (dealt out 48.5 us, but chains of 25 and 31 tiles instead of 27 and 4.24e-6).
 template <int TN>
 __global__ void __launch_bounds__(128)
 conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmz, int H, int W,
-                   int C, int cout, int tiles_x, int tiles_y, int ntiles, int nbk, int split, int per,
-                   int planes, int nstages, int stage_bytes, float alpha, float *gw, int ldg, int *err)
+                   int C, int cout, int tiles_x, int tiles_y, int ntiles, int nbk, int split0, int per0, int per1,
+                   int share, int planes, int nstages, int stage_bytes, float alpha, float *gw, int ldg, int *err)
 {
     extern __shared__ unsigned char dyn_raw[];
     __shared__ __align__(8) unsigned long long full[kWgStages], empty[kWgStages], done;
@@ -512,10 +513,11 @@ conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constan
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int mb = blockIdx.x / nbk, nb = blockIdx.x % nbk;
-    // CTAs [0, split) of a channel block are of the first kind
-    const bool second = (int)blockIdx.y >= split;
+    // CTAs [0, split0) of a channel block are of the first kind
+    const bool second = TN == 64 && (int)blockIdx.y >= split0;
     const int tap0 = second ? 4 : 0, tap1 = TN == 64 ? tap0 + 5 : 9;
-    const int t_beg = ((int)blockIdx.y - (second ? split : 0)) * per;
+    const int per = second ? per1 : per0;
+    const int t_beg = ((int)blockIdx.y - (second ? split0 : 0)) * per;
     const int t_end = min(ntiles, t_beg + per);
     if (t_beg >= t_end) return;             // uniform over the CTA
     const int a_bytes = (planes * kPlane + 127) / 128 * 128;
@@ -524,8 +526,8 @@ conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constan
 
     const uint32_t tmem = setup<kCols>(&tmem_holder, full, empty, &done, nstages, &failed);
     const int n_it = t_end - t_beg;
-    // tap 4 in its CTA's tiles [mid0, mid1); the other taps in all of them
-    const int half = (n_it + 1) / 2, mid0 = second ? half : 0, mid1 = (TN == 64 && !second) ? half : n_it;
+    // the first kind's tiles before `half` and the second kind's from there on have tap 4
+    const int half = share ? (n_it + 1) / 2 : n_it;
 
     if (warp == 0 && lane == 0) {
         asm volatile("prefetch.tensormap [%0];" :: "l"(reinterpret_cast<uint64_t>(&tmx)) : "memory");
@@ -548,10 +550,10 @@ conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constan
             if (!wait_or_fail(smem_u32(&full[s]), (uint32_t)((it / nstages) & 1), &failed, err)) break;
             asm volatile("tcgen05.fence::after_thread_sync;");
             const uint32_t st = base + (uint32_t)(s * stage_bytes);
+            const int ta = second && it < half ? 5 : tap0, tb = TN == 64 && !second && it >= half ? 4 : tap1;
             #pragma unroll 1
-            for (int t = tap0; t < tap1; ++t) {
-                if (t == 4 && (it < mid0 || it >= mid1)) continue;
-                const int ky = t / 3, kx = t % 3, it0 = t == 4 ? mid0 : 0;
+            for (int t = ta; t < tb; ++t) {
+                const int ky = t / 3, kx = t % 3, it0 = second && t == 4 ? half : 0;
                 #pragma unroll
                 for (int j = 0; j < kTileRows / 2; ++j) {        // K = 16 pixels: image rows 2j, 2j + 1
                     mma_f16(tmem + (uint32_t)((t - tap0) * TN),
@@ -573,7 +575,7 @@ conv3_wgrad_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constan
         const int c = kWgPlanes * 8 * mb + warp * 32 + lane;
         #pragma unroll 1
         for (int t = tap0; t < tap1; ++t) {
-            if (t == 4 && mid0 >= mid1) continue;
+            if (second && t == 4 && half >= n_it) continue;
             #pragma unroll 1
             for (int o0 = 0; o0 < TN; o0 += 32) {
                 uint32_t r[32];
@@ -1307,11 +1309,20 @@ extern "C" int smrt_nn_conv3_wgrad_tma(const void *xb, int N, int H, int W, int 
     const int mbk = (C + 8 * kWgPlanes - 1) / (8 * kWgPlanes), nbk = (cout + TN - 1) / TN;
     // one CTA per SM (each holds all 512 TMEM columns): split the pixel tiles to fill the SMs
     const int kinds = TN == 64 ? 2 : 1;
-    long long split = sm_count() / (mbk * nbk * kinds);
-    if (split < 1) split = 1;
-    if (split > ntiles) split = ntiles;
-    const int per = (int)((ntiles + split - 1) / split);
-    split = (ntiles + per - 1) / per;
+    const long long splits = std::max(sm_count() / (mbk * nbk), kinds);
+    auto tiles_per = [&](long long n) { return (int)((ntiles + std::min(n, ntiles) - 1) / std::min(n, ntiles)); };
+    long long split0 = splits, split1 = 0;
+    int per0 = tiles_per(split0), per1 = 1, share = 0;
+    if (TN == 64) {
+        const int most = tiles_per(std::max(sm_count() / (mbk * ((cout + kWgTN - 1) / kWgTN)), 1));
+        split0 = (5 * splits + 4) / 9;
+        per0 = tiles_per(split0);
+        per1 = tiles_per(splits - split0);
+        share = per0 > most || per1 > most;
+        if (share) per0 = per1 = tiles_per(splits / 2);
+        split1 = (ntiles + per1 - 1) / per1;
+    }
+    split0 = (ntiles + per0 - 1) / per0;
     const int a_bytes = (planes * kPlane + 127) / 128 * 128;
     const int stage = (a_bytes + TN / 8 * kDzPlane + 1023) / 1024 * 1024;
     const int a_reach = kWgPlanes * kPlane;         // the MMA's 128 rows read 16 planes from a stage start
@@ -1320,7 +1331,7 @@ extern "C" int smrt_nn_conv3_wgrad_tma(const void *xb, int N, int H, int W, int 
     while (nstages > 2 && need(nstages) + 1024 > 220 * 1024) --nstages;
     size_t smem = need(nstages) + 1024;
     if (smem < 120 * 1024) smem = 120 * 1024;       // keeps a second CTA (and its TMEM request) off the SM
-    if (smem > 220 * 1024 || mbk * nbk > 65535 || split * kinds > 65535)
+    if (smem > 220 * 1024 || mbk * nbk > 65535 || split0 + split1 > 65535)
         return tma_fail(SMRT_ERR_ARG, "smrt_nn_conv3_wgrad_tma: sizes out of range (C %d cout %d)", C, cout);
     auto kernel = TN == 64 ? conv3_wgrad_kernel<64> : conv3_wgrad_kernel<32>;
     static bool attr_set[2] = {false, false};
@@ -1329,9 +1340,9 @@ extern "C" int smrt_nn_conv3_wgrad_tma(const void *xb, int N, int H, int W, int 
         if (e != cudaSuccess) return tma_fail(SMRT_ERR_CUDA, "smrt_nn_conv3_wgrad_tma: %s", cudaGetErrorString(e));
         attr_set[kinds - 1] = true;
     }
-    dim3 grid(mbk * nbk, (unsigned)(split * kinds));
+    dim3 grid(mbk * nbk, (unsigned)(split0 + split1));
     kernel<<<grid, 128, smem, (cudaStream_t)stream>>>(tmx, tmz, H, W, C, cout, tiles_x, tiles_y, (int)ntiles, nbk,
-                                                      (int)split, per, planes, nstages, stage, alpha, gw, ldg,
+                                                      (int)split0, per0, per1, share, planes, nstages, stage, alpha, gw, ldg,
                                                       err);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return tma_fail(SMRT_ERR_CUDA, "smrt_nn_conv3_wgrad_tma: %s", cudaGetErrorString(e));
