@@ -409,13 +409,13 @@ __device__ __forceinline__ void pull_canonical(const typename Prec<PREC>::R *sta
     }
 }
 
-// Where f_a of a node whose nine source nodes lie inside the lattice (no wall, no wrap) is stored.
+// Where f_a of a node whose nine source nodes lie inside the lattice (no wall, no wrap) is stored, from the node's place
+// in the first population.
 template <int MODE, class C>
-__device__ __forceinline__ size_t inner_at(const Params<C> &p, int a, int i, int j)
+__device__ __forceinline__ long long inner_off(const Params<C> &p, int a)
 {
-    const long long node = (long long)j * p.pitch + i;
-    if (MODE == MODE_AA_EVEN) return (size_t)(a * p.plane + node);
-    return (size_t)((MODE == MODE_AB ? a : opp(a)) * p.plane + node - (ey(a) * p.pitch + ex(a)));
+    return MODE == MODE_AA_EVEN ? (long long)a * p.plane
+                                : (long long)(MODE == MODE_AB ? a : opp(a)) * p.plane - (long long)ey(a) * p.pitch - ex(a);
 }
 
 // pull_canonical for such a node.
@@ -424,8 +424,9 @@ __device__ __forceinline__ void pull_inner(const typename Prec<PREC>::R *state, 
                                            int i, int j, typename Prec<PREC>::C g[9])
 {
     using P = Prec<PREC>;
+    const typename P::R *s0 = state + (size_t)j * (size_t)p.pitch + (size_t)i;
     #pragma unroll
-    for (int a = 0; a < 9; ++a) g[a] = P::to_c(state[inner_at<MODE>(p, a, i, j)]);
+    for (int a = 0; a < 9; ++a) g[a] = P::to_c(s0[inner_off<MODE>(p, a)]);
 }
 
 template <int PREC, int MODE>
@@ -472,7 +473,7 @@ __device__ __forceinline__ void init_store_f(typename Prec<PREC>::R *state, cons
     const float eu = float(ex(A)) * ux + float(ey(A)) * uy;
     float g = WeightMul<float>::template mul<A>(drho + d * (3.0f * eu + 4.5f * eu * eu - 1.5f * uu));
     if constexpr (INNER) {
-        state[inner_at<MODE>(p, A, i, j)] = P::to_r(g);
+        state[(long long)j * p.pitch + i + inner_off<MODE>(p, A)] = P::to_r(g);
     } else {
         const Loc L = pull_loc<MODE>(p, A, i, j);
         if (L.side >= 0) g -= p.corr[L.side][A];
