@@ -255,15 +255,41 @@ __global__ void add_vec(const float *a, const float *b, int n4, float *y)
 
 // 1x1 convolution with few outputs (the network's head), float32 on the CUDA cores: a product of
 // COUT x C per pixel is far too narrow for the tensor cores and is bound by reading x.
-// Forward: y[p][o] = sum_c x[p][c] w[o][c] + b[o].  Thread: one pixel, its channels summed in order.  A block
-// stages its 256 pixels in shared memory with coalesced 16-byte loads, 32 channels at a time (a thread that
-// reads its own pixel from memory touches a line of its own with every load: 43 us at 16 x 256^2 x 32, whose
-// bytes take 22; staged: 32 us).
+// Forward: y[p][o] = sum_c x[p][c] w[o][c] + b[o].  Thread: one pixel, its channels summed in order.
+template <int COUT>
+__global__ void __launch_bounds__(256)
+conv1x1_small(const float *__restrict__ x, int P, int C, const float *__restrict__ w, const float *__restrict__ bias,
+              float *__restrict__ y)
+{
+    __shared__ float sw[COUT * 64];
+    for (int i = threadIdx.x; i < COUT * C; i += blockDim.x) sw[i] = w[i];
+    __syncthreads();
+    for (unsigned p = blockIdx.x * blockDim.x + threadIdx.x; p < (unsigned)P; p += gridDim.x * blockDim.x) {
+        float acc[COUT];
+        #pragma unroll
+        for (int o = 0; o < COUT; ++o) acc[o] = bias ? bias[o] : 0.0f;
+        const float *xp = x + (size_t)p * C;
+        for (int c = 0; c < C; c += 4) {
+            const Vec<4> v = ldv<4>(xp + c);
+            #pragma unroll
+            for (int o = 0; o < COUT; ++o)
+                #pragma unroll
+                for (int i = 0; i < 4; ++i) acc[o] = fmaf(v.v[i], sw[o * C + c + i], acc[o]);
+        }
+        #pragma unroll
+        for (int o = 0; o < COUT; ++o) y[(size_t)p * COUT + o] = acc[o];
+    }
+}
+
+// The same for 32 or 64 channels, where the pixels of a warp start a whole number of 128-byte lines apart and reading
+// them pixel by pixel leaves most of the cache unused: a block stages its 256 pixels in shared memory with coalesced
+// 16-byte loads, 32 channels at a time.  1 M pixels, three outputs, us pixel by pixel / staged: 32 channels 43 / 32,
+// 64 79 / 58; but 20 channels 16.8 / 24.4, 12 channels 11 / 18.
 constexpr int kHeadBX = 256, kHeadC = 32;
 template <int COUT>
 __global__ void __launch_bounds__(kHeadBX)
-conv1x1_small(const float *__restrict__ x, int P, int C, const float *__restrict__ w, const float *__restrict__ bias,
-              float *__restrict__ y)
+conv1x1_small_staged(const float *__restrict__ x, int P, int C, const float *__restrict__ w,
+                     const float *__restrict__ bias, float *__restrict__ y)
 {
     __shared__ __align__(16) float sx[kHeadBX * (kHeadC + 1)];
     __shared__ float sw[COUT * 64];
@@ -467,14 +493,20 @@ cudaError_t vec_upcat_bwd(const float *dy, int N, int H, int W, int Ca, int Cb, 
     return cudaGetLastError();
 }
 
+template <int COUT>
+void launch_head(const float *x, long long P, int C, const float *w, const float *bias, float *y, cudaStream_t s)
+{
+    if (C % kHeadC == 0) conv1x1_small_staged<COUT><<<blocks_for(P), kHeadBX, 0, s>>>(x, (int)P, C, w, bias, y);
+    else conv1x1_small<COUT><<<blocks_for(P), 256, 0, s>>>(x, (int)P, C, w, bias, y);
+}
+
 cudaError_t small_conv1x1(const float *x, long long P, int C, const float *w, const float *bias, int cout, float *y,
                           cudaStream_t s)
 {
-    const unsigned blocks = blocks_for(P);
     switch (cout) {
-    case 1: conv1x1_small<1><<<blocks, kHeadBX, 0, s>>>(x, (int)P, C, w, bias, y); break;
-    case 2: conv1x1_small<2><<<blocks, kHeadBX, 0, s>>>(x, (int)P, C, w, bias, y); break;
-    default: conv1x1_small<3><<<blocks, kHeadBX, 0, s>>>(x, (int)P, C, w, bias, y); break;
+    case 1: launch_head<1>(x, P, C, w, bias, y, s); break;
+    case 2: launch_head<2>(x, P, C, w, bias, y, s); break;
+    default: launch_head<3>(x, P, C, w, bias, y, s); break;
     }
     return cudaGetLastError();
 }
