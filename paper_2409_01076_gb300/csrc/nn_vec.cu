@@ -330,18 +330,19 @@ conv1x1_small_staged(const float *__restrict__ x, int P, int C, const float *__r
 // 8 warps per SM: 96 us at 16 x 256^2 x 32, whose bytes take 41; by quads: 57 us).  A block adds its sums in
 // shared memory and then into dw / db with one atomic per entry.  That last sum, block after block onto one float,
 // is where the rounding errors of dw and db come from, so the blocks are large and few: one per SM (error of dw against
-// 64 bits 1.9e-7 there; with 8 blocks of 256 threads per SM 5.3e-7).  C <= 64; the block is a multiple of C / 4.
+// 64 bits 1.9e-7 there; with 8 blocks of 256 threads per SM 5.3e-7).  C <= 64.
 template <int COUT> struct HeadBwd { static constexpr int BX = 1024, per_sm = 1; };
 template <> struct HeadBwd<1> { static constexpr int BX = 640, per_sm = 2; };       // fewer registers, more threads
 template <int COUT>
 __global__ void __launch_bounds__(HeadBwd<COUT>::BX, HeadBwd<COUT>::per_sm)
-conv1x1_small_bwd(const float *__restrict__ dy, const float *__restrict__ x, int P, int C,
+conv1x1_small_bwd(const float *__restrict__ dy, const float *__restrict__ x, int P, int C, int L,
                   const float *__restrict__ w, float *__restrict__ dx, float *dw, float *db)
 {
     __shared__ float sacc[COUT * 64 + COUT];
     for (int i = threadIdx.x; i < COUT * C + COUT; i += blockDim.x) sacc[i] = 0.0f;
     __syncthreads();
-    const int Q = C / 4, q = threadIdx.x % Q, per_block = blockDim.x / Q;
+    const int q = threadIdx.x % L, per_block = blockDim.x / L;
+    const bool has = 4 * q < C;
     float gw[COUT][4], gb[COUT], wq[COUT][4];
     #pragma unroll
     for (int o = 0; o < COUT; ++o) {
@@ -349,12 +350,12 @@ conv1x1_small_bwd(const float *__restrict__ dy, const float *__restrict__ x, int
         #pragma unroll
         for (int i = 0; i < 4; ++i) {
             gw[o][i] = 0.0f;
-            wq[o][i] = w[o * C + 4 * q + i];
+            wq[o][i] = has ? w[o * C + 4 * q + i] : 0.0f;
         }
     }
     constexpr int kInFlight = COUT == 1 ? 4 : 2;
     #pragma unroll kInFlight
-    for (unsigned p = blockIdx.x * per_block + threadIdx.x / Q; p < (unsigned)P; p += gridDim.x * per_block) {
+    for (unsigned p = has ? blockIdx.x * per_block + threadIdx.x / L : P; p < (unsigned)P; p += gridDim.x * per_block) {
         float g[COUT];
         #pragma unroll
         for (int o = 0; o < COUT; ++o) {
@@ -375,12 +376,10 @@ conv1x1_small_bwd(const float *__restrict__ dy, const float *__restrict__ x, int
         }
         if (dx) stv<4>(dx + (size_t)p * C + 4 * q, d);
     }
-    // a warp's lanes of one quad first (Q a power of two: whole warps), then one shared-memory atomic per warp and entry
-    const bool lanes = (Q & (Q - 1)) == 0;
-    const bool adds = !lanes || (threadIdx.x & 31) < Q;
+    // a warp's lanes of one quad first where L is a power of two, then one shared-memory atomic per warp and entry
+    const bool shuffles = (L & (L - 1)) == 0, adds = has && (!shuffles || (threadIdx.x & 31) < L);
     auto warp_quad = [&](float v) {
-        if (lanes)
-            for (int o = 16; o >= Q; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        for (int o = 16; shuffles && o >= L; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         return v;
     };
     #pragma unroll
@@ -515,10 +514,15 @@ template <int COUT>
 void launch_head_bwd(const float *dy, const float *x, long long P, int C, const float *w, float *dx, float *dw, float *db,
                      cudaStream_t s)
 {
-    const int threads = HeadBwd<COUT>::BX / (C / 4) * (C / 4);
     long long b = (P + 127) / 128;                      // few pixels: at least 128 to a block
     if (b > 152LL * HeadBwd<COUT>::per_sm) b = 152LL * HeadBwd<COUT>::per_sm;
-    conv1x1_small_bwd<COUT><<<(unsigned)b, threads, 0, s>>>(dy, x, (int)P, C, w, dx, dw, db);
+    // Lanes to a pixel: its quads, or the next power of two (the lanes beyond idle), so that a warp's lanes of one quad
+    // add up by shuffles.  Without them the block's last sums take 5 us, 30 where few entries take them all (C = 12):
+    // worth it for many pixels whose idle lanes would cost more (C = 20, one output, 4 M pixels 121 / 140 us).
+    int L = C / 4;
+    if (L < 5 || P < (1 << 18))
+        while (L & (L - 1)) ++L;
+    conv1x1_small_bwd<COUT><<<(unsigned)b, HeadBwd<COUT>::BX / L * L, 0, s>>>(dy, x, (int)P, C, L, w, dx, dw, db);
 }
 
 cudaError_t small_conv1x1_bwd(const float *dy, const float *x, long long P, int C, const float *w, int cout, float *dx,
