@@ -250,7 +250,7 @@ __device__ __forceinline__ void sweep(const typename Prec<PREC>::R *__restrict__
             #pragma unroll
             for (int a = 1; a < 9; ++a) {
                 if (ex(a) == 0) continue;
-                // the order of SweepState::el; a link through the bottom or top wall is that wall's
+                // the order of `wall` (SweepShared); a link through the bottom or top wall is that wall's
                 const bool here = (ex(a) > 0 ? at_left : at_right) && !((ey(a) > 0 && b) || (ey(a) < 0 && t));
                 const int x = ey(a) == 0 ? 0 : ey(a) > 0 ? 1 : 2;
                 if (here) {
